@@ -75,17 +75,20 @@ __device__ __forceinline__ bool match_valid(const int32_t* __restrict__ m, long 
 
 __global__ void __launch_bounds__(kThreads) k_pnp_flags(const int32_t* __restrict__ m, long long n,
                                                         const float* __restrict__ alpha, int npix, float min_alpha,
-                                                        unsigned* __restrict__ blk, State* __restrict__ st) {
+                                                        unsigned* __restrict__ blk, unsigned* __restrict__ words,
+                                                        State* __restrict__ st) {
   __shared__ unsigned s_w[kThreads / 32];
   const long long base = (long long)blockIdx.x * kCompact;
   unsigned c = 0, nbad = 0;
+#pragma unroll
   for (int k = 0; k < kCompact / kThreads; ++k) {
     const long long i = base + k * kThreads + threadIdx.x;
-    if (i < n) {
-      bool bad;
-      c += match_valid(m, i, alpha, npix, min_alpha, &bad) ? 1u : 0u;
-      nbad += bad ? 1u : 0u;
-    }
+    bool bad = false;
+    const bool v = i < n && match_valid(m, i, alpha, npix, min_alpha, &bad);
+    c += v ? 1u : 0u;
+    nbad += bad ? 1u : 0u;
+    const unsigned b = __ballot_sync(0xffffffffu, v);
+    if ((threadIdx.x & 31) == 0) words[i >> 5] = b;  // validity bits, for the samples' ranks
   }
   c = __reduce_add_sync(0xffffffffu, c);
   nbad = __reduce_add_sync(0xffffffffu, nbad);
@@ -138,13 +141,31 @@ __global__ void __launch_bounds__(1024) k_pnp_scan(unsigned* __restrict__ blk, i
   if (tid == 0) st->n_valid = s_carry;
 }
 
+// World point of the rendered pixel rp (fp64). z = depth / alpha without a
+// division: the binary32 reciprocal refined by one Newton step (48 bits), then
+// one correction of the quotient.
+__device__ __forceinline__ void lift_point(const float* __restrict__ depth, const float* __restrict__ alpha, int rp,
+                                           const Cam& cam, const Pose12& Tr, double& X, double& Y, double& Z) {
+  const double A = alpha[rp], D = depth[rp];
+  double rcp = (double)(1.0f / alpha[rp]);
+  rcp = rcp * (2.0 - A * rcp);
+  double z = D * rcp;
+  z = fma(rcp, fma(-z, A, D), z);
+  const double xc = z * (((double)(rp % cam.W) + 0.5 - cam.cx) * cam.ifx);
+  const double yc = z * (((double)(rp / cam.W) + 0.5 - cam.cy) * cam.ify);
+  const double d0 = xc - Tr.v[9], d1 = yc - Tr.v[10], d2 = z - Tr.v[11];
+  const double* R = Tr.v;
+  X = R[0] * d0 + R[3] * d1 + R[6] * d2;  // R^T d
+  Y = R[1] * d0 + R[4] * d1 + R[7] * d2;
+  Z = R[2] * d0 + R[5] * d1 + R[8] * d2;
+}
+
 __global__ void __launch_bounds__(kThreads) k_pnp_lift(const int32_t* __restrict__ m, long long n,
                                                        const float* __restrict__ depth,
                                                        const float* __restrict__ alpha, Cam cam, Pose12 Tr,
                                                        float min_alpha, const unsigned* __restrict__ blk,
                                                        double* __restrict__ X64, float4* __restrict__ X32,
-                                                       float2* __restrict__ nab, float2* __restrict__ pix,
-                                                       int32_t* __restrict__ vidx) {
+                                                       float2* __restrict__ nab, int32_t* __restrict__ vidx) {
   __shared__ unsigned s_w[kThreads / 32];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const long long base = (long long)blockIdx.x * kCompact;
@@ -166,26 +187,13 @@ __global__ void __launch_bounds__(kThreads) k_pnp_lift(const int32_t* __restrict
     if (v) {
       const unsigned o = off + before + (unsigned)__popc(b & ((1u << lane) - 1u));
       const int qp = m[3 * i + 1], rp = m[3 * i + 2];
-      // z = depth / alpha in fp64 without a division: the binary32 reciprocal
-      // refined by one Newton step (48 bits), then one correction of the quotient
-      const double A = alpha[rp], D = depth[rp];
-      double rcp = (double)(1.0f / alpha[rp]);
-      rcp = rcp * (2.0 - A * rcp);
-      double z = D * rcp;
-      z = fma(rcp, fma(-z, A, D), z);
-      const double xc = z * (((double)(rp % cam.W) + 0.5 - cam.cx) * cam.ifx);
-      const double yc = z * (((double)(rp / cam.W) + 0.5 - cam.cy) * cam.ify);
-      const double d0 = xc - Tr.v[9], d1 = yc - Tr.v[10], d2 = z - Tr.v[11];
-      const double* R = Tr.v;
-      const double X = R[0] * d0 + R[3] * d1 + R[6] * d2;  // R^T d
-      const double Y = R[1] * d0 + R[4] * d1 + R[7] * d2;
-      const double Z = R[2] * d0 + R[5] * d1 + R[8] * d2;
+      double X, Y, Z;
+      lift_point(depth, alpha, rp, cam, Tr, X, Y, Z);
       X64[3 * (size_t)o] = X;
       X64[3 * (size_t)o + 1] = Y;
       X64[3 * (size_t)o + 2] = Z;
       X32[o] = make_float4((float)X, (float)Y, (float)Z, 0.0f);
       const double px = (double)(qp % cam.W) + 0.5, py = (double)(qp / cam.W) + 0.5;
-      pix[o] = make_float2((float)px, (float)py);
       nab[o] = make_float2((float)(-(px - cam.cx) * cam.ifx), (float)(-(py - cam.cy) * cam.ify));
       vidx[o] = (int32_t)i;
     }
@@ -203,8 +211,10 @@ __global__ void __launch_bounds__(kThreads) k_pnp_lift(const int32_t* __restrict
 // = 0 (for q = 0: y^2 = the roots of z^2 + p z + r). The closed form runs in a
 // few hundred fp64 operations, against thousands for bracketing: fp64 is slow
 // on this part. Each real root is then polished by two Newton steps on the
-// original quartic. Returns the count; roots ascending.
-__device__ int quartic_real_roots(const double* q4, double* out) {
+// original quartic. Called by the four lanes of a sample together: the closed
+// form is the same in each, root k is polished by lane k. Returns the count;
+// roots ascending, all four lanes holding all of them.
+__device__ int quartic_real_roots(const double* q4, double (&out)[4], int k, unsigned quad) {
   const double a = q4[3] / q4[4], b = q4[2] / q4[4], c = q4[1] / q4[4], d = q4[0] / q4[4];
   const double a2 = a * a;
   const double p = b - 0.375 * a2;
@@ -230,7 +240,7 @@ __device__ int quartic_real_roots(const double* q4, double* out) {
     const double f = ((m + A) * m + B) * m + C, df = (3.0 * m + 2.0 * A) * m + B;
     if (df != 0.0) m -= f / df;
   }
-  double y[4];
+  double y[4] = {0.0, 0.0, 0.0, 0.0};
   int ny = 0;
   const double s2 = 2.0 * m - p;
   if (s2 > 1e-14 * (fabs(p) + fabs(m) + 1e-300)) {
@@ -259,16 +269,15 @@ __device__ int quartic_real_roots(const double* q4, double* out) {
         }
     }
   }
-  int n = 0;
-  for (int k = 0; k < ny; ++k) {
-    double x = y[k] - 0.25 * a;
-    for (int it = 0; it < 2; ++it) {
-      const double f = (((x + a) * x + b) * x + c) * x + d;
-      const double df = ((4.0 * x + 3.0 * a) * x + 2.0 * b) * x + c;
-      if (df != 0.0) x -= f / df;
-    }
-    out[n++] = x;
+  double x = (k == 0 ? y[0] : k == 1 ? y[1] : k == 2 ? y[2] : y[3]) - 0.25 * a;
+  for (int it = 0; it < 2; ++it) {
+    const double f = (((x + a) * x + b) * x + c) * x + d;
+    const double df = ((4.0 * x + 3.0 * a) * x + 2.0 * b) * x + c;
+    if (df != 0.0) x -= f / df;
   }
+  const int n = ny;
+#pragma unroll
+  for (int r = 0; r < 4; ++r) out[r] = __shfl_sync(quad, x, r, 4);
   for (int i = 1; i < n; ++i)  // ascending (insertion sort, n <= 4)
     for (int j = i; j > 0 && out[j - 1] > out[j]; --j) {
       const double tmp = out[j];
@@ -297,40 +306,74 @@ __device__ void frame3(const double* P0, const double* P1, const double* P2, dou
   }
 }
 
-__global__ void __launch_bounds__(32) k_pnp_p3p(const double* __restrict__ X64, const float2* __restrict__ pix,
-                                                 const State* __restrict__ st, const uint32_t* __restrict__ words,
-                                                 int n_hyp, Cam cam, double* __restrict__ poses64,
-                                                 float4* __restrict__ poses32, int* __restrict__ counts) {
-  const int h = blockIdx.x * blockDim.x + threadIdx.x;
-  if (h >= n_hyp) return;
+// Match index of the valid match of rank `idx` (in match order): the block whose
+// exclusive count holds it, then its validity bits.
+__device__ long long nth_valid(unsigned idx, const unsigned* __restrict__ blk, int nb,
+                               const unsigned* __restrict__ words) {
+  int lo = 0, hi = nb - 1;  // last block whose first rank is <= idx
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (blk[mid] <= idx) lo = mid; else hi = mid - 1;
+  }
+  unsigned rem = idx - blk[lo];
+  const uint4* w4 = reinterpret_cast<const uint4*>(words + (size_t)lo * (kCompact / 32));
+  unsigned word = 0;
+  int at = -1;
 #pragma unroll
-  for (int s = 0; s < kSol; ++s) counts[kSol * h + s] = -1;
-  const unsigned long long K = st->n_valid;
-  if (K < 3) return;
-  int idx[3];
-  for (int k = 0; k < 3; ++k) idx[k] = (int)(((unsigned long long)words[3 * h + k] * K) >> 32);
-  if (idx[0] == idx[1] || idx[0] == idx[2] || idx[1] == idx[2]) return;
+  for (int q = 0; q < kCompact / 128; ++q) {
+    const uint4 v = w4[q];
+    const unsigned u[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      const unsigned c = (unsigned)__popc(u[e]);
+      if (at < 0) {
+        if (rem < c) {
+          at = 4 * q + e;
+          word = u[e];
+        } else {
+          rem -= c;
+        }
+      }
+    }
+  }
+  for (; rem > 0; --rem) word &= word - 1;  // at >= 0: the block holds the rank
+  return (long long)lo * kCompact + 32 * at + (__ffs(word) - 1);
+}
+
+// This lane's solution of one sample (root `lane4` of the quartic), called by the
+// sample's four lanes together; false when there is none.
+__device__ bool p3p_lane(const int32_t* __restrict__ m, const float* __restrict__ depth,
+                         const float* __restrict__ alpha, const unsigned* __restrict__ blk,
+                         const unsigned* __restrict__ vwords, int nb, unsigned long long K,
+                         const uint32_t* __restrict__ w3, const Cam& cam, const Pose12& Tr, int lane4, unsigned quad,
+                         double (&R)[9], double (&tt)[3]) {
+  if (K < 3) return false;
+  unsigned idx[3];
+  for (int k = 0; k < 3; ++k) idx[k] = (unsigned)(((unsigned long long)w3[k] * K) >> 32);
+  if (idx[0] == idx[1] || idx[0] == idx[2] || idx[1] == idx[2]) return false;
   double X[3][3], f[3][3];
   for (int k = 0; k < 3; ++k) {
-    for (int a = 0; a < 3; ++a) X[k][a] = X64[3 * (size_t)idx[k] + a];
-    const float2 p = pix[idx[k]];
+    const long long i = nth_valid(idx[k], blk, nb, vwords);
+    const int qp = m[3 * i + 1], rp = m[3 * i + 2];
+    lift_point(depth, alpha, rp, cam, Tr, X[k][0], X[k][1], X[k][2]);
+    const float2 p = make_float2((float)((double)(qp % cam.W) + 0.5), (float)((double)(qp / cam.W) + 0.5));
     const double bx = ((double)p.x - cam.cx) / cam.fx, by = ((double)p.y - cam.cy) / cam.fy;
-    const double nb = sqrt(bx * bx + by * by + 1.0);
-    f[k][0] = bx / nb;
-    f[k][1] = by / nb;
-    f[k][2] = 1.0 / nb;
+    const double nb2 = sqrt(bx * bx + by * by + 1.0);
+    f[k][0] = bx / nb2;
+    f[k][1] = by / nb2;
+    f[k][2] = 1.0 / nb2;
   }
   auto d2 = [&](int i, int j) {
     const double a = X[i][0] - X[j][0], b = X[i][1] - X[j][1], c = X[i][2] - X[j][2];
     return a * a + b * b + c * c;
   };
   const double a2 = d2(1, 2), b2 = d2(0, 2), c2 = d2(0, 1);
-  if (!(a2 > 0.0 && b2 > 0.0 && c2 > 0.0)) return;
+  if (!(a2 > 0.0 && b2 > 0.0 && c2 > 0.0)) return false;
   {  // collinear world points
     const double u[3] = {X[1][0] - X[0][0], X[1][1] - X[0][1], X[1][2] - X[0][2]};
     const double w[3] = {X[2][0] - X[0][0], X[2][1] - X[0][1], X[2][2] - X[0][2]};
     const double cx = u[1] * w[2] - u[2] * w[1], cy = u[2] * w[0] - u[0] * w[2], cz = u[0] * w[1] - u[1] * w[0];
-    if (sqrt(cx * cx + cy * cy + cz * cz) <= 1e-12 * (a2 + b2 + c2)) return;
+    if (sqrt(cx * cx + cy * cy + cz * cz) <= 1e-12 * (a2 + b2 + c2)) return false;
   }
   const double ca = f[1][0] * f[2][0] + f[1][1] * f[2][1] + f[1][2] * f[2][2];
   const double cb = f[0][0] * f[2][0] + f[0][1] * f[2][1] + f[0][2] * f[2][2];
@@ -347,43 +390,66 @@ __global__ void __launch_bounds__(32) k_pnp_p3p(const double* __restrict__ X64, 
     for (int j = 0; j < 3; ++j) Q[i + j] += 4.0 * D2[i] * E[j] + N[i] * N[j];
   for (int i = 0; i < 3; ++i)
     for (int j = 0; j < 2; ++j) Q[i + j] -= 4.0 * cg * N[i] * D[j];
-  if (Q[4] == 0.0) return;
+  if (Q[4] == 0.0) return false;
   double roots[4];
-  const int nr = quartic_real_roots(Q, roots);
-  int ns = 0;
+  const int nr = quartic_real_roots(Q, roots, lane4, quad);
   double FX[3][3];
   bool okx;
   frame3(X[0], X[1], X[2], FX, &okx);
-  if (!okx) return;
-  for (int r = 0; r < nr && ns < kSol; ++r) {
-    const double v = roots[r];
-    if (!(v > 0.0)) continue;
+  if (!okx) return false;
+  // lane r: the pose of root r
+  const double v = lane4 == 0 ? roots[0] : lane4 == 1 ? roots[1] : lane4 == 2 ? roots[2] : roots[3];
+  bool ok = lane4 < nr && v > 0.0;
+  if (ok) {
     const double Dv = D[0] + D[1] * v;
-    if (Dv == 0.0) continue;
+    ok = Dv != 0.0;
     const double u = (N[0] + v * (N[1] + v * N[2])) / (2.0 * Dv);
-    if (!(u > 0.0)) continue;
-    const double s1 = sqrt(b2 / (1.0 + v * v - 2.0 * v * cb));
-    const double s[3] = {s1, u * s1, v * s1};
-    double Qc[3][3];
-    for (int i = 0; i < 3; ++i)
-      for (int a = 0; a < 3; ++a) Qc[i][a] = s[i] * f[i][a];
-    double FQ[3][3];
-    bool okq;
-    frame3(Qc[0], Qc[1], Qc[2], FQ, &okq);
-    if (!okq) continue;
-    double R[9], t[3];
-    for (int i = 0; i < 3; ++i)
-      for (int j = 0; j < 3; ++j) R[3 * i + j] = FQ[i][0] * FX[j][0] + FQ[i][1] * FX[j][1] + FQ[i][2] * FX[j][2];
-    for (int i = 0; i < 3; ++i)
-      t[i] = Qc[0][i] - (R[3 * i] * X[0][0] + R[3 * i + 1] * X[0][1] + R[3 * i + 2] * X[0][2]);
-    double* o = poses64 + ((size_t)kSol * h + ns) * kPose;
-    for (int q = 0; q < 9; ++q) o[q] = R[q];
-    for (int q = 0; q < 3; ++q) o[9 + q] = t[q];
-    float4* o32 = poses32 + ((size_t)kSol * h + ns) * 3;
-    for (int i = 0; i < 3; ++i) o32[i] = make_float4((float)R[3 * i], (float)R[3 * i + 1], (float)R[3 * i + 2], (float)t[i]);
-    counts[kSol * h + ns] = 0;
-    ++ns;
+    ok = ok && u > 0.0;
+    if (ok) {
+      const double s1 = sqrt(b2 / (1.0 + v * v - 2.0 * v * cb));
+      const double s[3] = {s1, u * s1, v * s1};
+      double Qc[3][3];
+      for (int i = 0; i < 3; ++i)
+        for (int a = 0; a < 3; ++a) Qc[i][a] = s[i] * f[i][a];
+      double FQ[3][3];
+      frame3(Qc[0], Qc[1], Qc[2], FQ, &ok);
+      if (ok) {
+        for (int i = 0; i < 3; ++i)
+          for (int j = 0; j < 3; ++j) R[3 * i + j] = FQ[i][0] * FX[j][0] + FQ[i][1] * FX[j][1] + FQ[i][2] * FX[j][2];
+        for (int i = 0; i < 3; ++i)
+          tt[i] = Qc[0][i] - (R[3 * i] * X[0][0] + R[3 * i + 1] * X[0][1] + R[3 * i + 2] * X[0][2]);
+      }
+    }
   }
+  return ok;
+}
+
+// Four lanes per sample. The chain of dependent fp64 operations of one sample is
+// the whole time, so its up to four roots are polished and turned into poses
+// side by side. The three points are lifted here as k_pnp_lift lifts them, so
+// that this kernel needs the compaction's counts only and runs beside it.
+// 53 us for 128 samples beside 50 us of lifting 490,000 matches; after it, with
+// a thread per sample, it took 55 us more.
+__global__ void __launch_bounds__(32) k_pnp_p3p(const int32_t* __restrict__ m, const float* __restrict__ depth,
+                                                const float* __restrict__ alpha, const unsigned* __restrict__ blk,
+                                                const unsigned* __restrict__ vwords, int nb,
+                                                const State* __restrict__ st, const uint32_t* __restrict__ words,
+                                                int n_hyp, Cam cam, Pose12 Tr, double* __restrict__ poses64,
+                                                float4* __restrict__ poses32, int* __restrict__ counts) {
+  const int t = blockIdx.x * blockDim.x + threadIdx.x, h = t / kSol, lane4 = t % kSol;
+  if (h >= n_hyp) return;  // whole quads
+  const unsigned quad = 0xfu << (threadIdx.x & 28);
+  double R[9], tt[3];
+  const bool ok = p3p_lane(m, depth, alpha, blk, vwords, nb, st->n_valid, words + 3 * (size_t)h, cam, Tr, lane4, quad, R, tt);
+  const unsigned found = __ballot_sync(quad, ok) >> (threadIdx.x & 28);
+  counts[kSol * h + lane4] = lane4 < __popc(found) ? 0 : -1;
+  if (!ok) return;
+  const int ns = __popc(found & ((1u << lane4) - 1u));  // solutions in root order
+  double* o = poses64 + ((size_t)kSol * h + ns) * kPose;
+  for (int q = 0; q < 9; ++q) o[q] = R[q];
+  for (int q = 0; q < 3; ++q) o[9 + q] = tt[q];
+  float4* o32 = poses32 + ((size_t)kSol * h + ns) * 3;
+  for (int i = 0; i < 3; ++i) o32[i] = make_float4((float)R[3 * i], (float)R[3 * i + 1], (float)R[3 * i + 2], (float)tt[i]);
 }
 
 // ------------------------------------------------------------------ scoring (fp32, packed pairs)
@@ -567,10 +633,87 @@ __global__ void __launch_bounds__(kThreads) k_pnp_gn(const float4* __restrict__ 
   }
 }
 
-// Left update T <- Exp(xi) T (Rodrigues; V = I + b [phi]x + c [phi]x^2 on rho).
-__device__ void se3_left(const double xi[6], double T[kPose]) {
-  const double* w = xi + 3;
-  const double t2 = w[0] * w[0] + w[1] * w[1] + w[2] * w[2];
+constexpr int kSolveParts = 8;  // partial sums per component in the solve kernel
+
+// One Gauss-Newton update. The partials of a component's part are loaded all at
+// once, then added in order; the 6 x 6 system is solved by one warp, lane i
+// holding row i, so that a column's rows, and the 3 x 3 entries of the left
+// update T <- Exp(xi) T (Rodrigues; V = I + b [phi]x + c [phi]x^2 on rho), are
+// computed side by side: the serial chain of fp64 operations is the whole time.
+// 10.5 us a step (14.6 us with one thread for the system and the update).
+__global__ void __launch_bounds__(kGnVals * kSolveParts) k_pnp_gn_solve(const double* __restrict__ partials,
+                                                                         State* __restrict__ st) {
+  static_assert(kGnBlocks % kSolveParts == 0, "equal parts");
+  __shared__ double part[kGnVals][kSolveParts];
+  __shared__ double s[kGnVals];
+  if (!st->active) return;
+  {  // component k, blocks j, j + 8, ... in order; then the 8 parts in order
+    const int k = threadIdx.x / kSolveParts, j = threadIdx.x % kSolveParts;
+    constexpr int kN = kGnBlocks / kSolveParts;
+    double v[kN];
+#pragma unroll
+    for (int i = 0; i < kN; ++i) v[i] = partials[(size_t)(j + kSolveParts * i) * kGnVals + k];
+    double a = 0.0;
+#pragma unroll
+    for (int i = 0; i < kN; ++i) a += v[i];
+    part[k][j] = a;
+  }
+  __syncthreads();
+  if (threadIdx.x < kGnVals) {
+    double a = 0.0;
+    for (int j = 0; j < kSolveParts; ++j) a += part[threadIdx.x][j];
+    s[threadIdx.x] = a;
+  }
+  __syncthreads();
+  if (threadIdx.x >= 32) return;
+  if (s[27] < 3.0) {
+    if (threadIdx.x == 0) st->active = 0;
+    return;
+  }
+  const int lane = threadIdx.x;
+  const int row = lane < 6 ? lane : 5;  // the other lanes repeat row 5
+  double H[6], L[6];
+#pragma unroll
+  for (int c = 0; c < 6; ++c) {
+    const int lo = row < c ? row : c, hi = row < c ? c : row;
+    H[c] = s[lo * 6 - lo * (lo - 1) / 2 + hi - lo];  // upper triangle by rows
+    L[c] = 0.0;
+  }
+  // Cholesky H = L L^T with the reciprocal diagonal: one reciprocal square
+  // root per column and multiplications (fp64 division is a long sequence here)
+  double inv[6];
+#pragma unroll
+  for (int j = 0; j < 6; ++j) {
+    double e = H[j];  // rows i > j: the entry; row j: the pivot
+#pragma unroll
+    for (int m = 0; m < j; ++m) e -= L[m] * __shfl_sync(0xffffffffu, L[m], j);
+    const double d = __shfl_sync(0xffffffffu, e, j);
+    if (!(d > 0.0)) {
+      if (lane == 0) st->active = 0;
+      return;
+    }
+    inv[j] = rsqrt(d);
+    L[j] = e * inv[j];
+  }
+  double y[6], xi[6];
+  {
+    double e = -s[21 + row];  // L y = -g
+#pragma unroll
+    for (int i = 0; i < 6; ++i) {
+      y[i] = __shfl_sync(0xffffffffu, e, i) * inv[i];
+      e -= L[i] * y[i];
+    }
+  }
+#pragma unroll
+  for (int i = 5; i >= 0; --i) {  // L^T xi = y
+    double e = y[i];
+#pragma unroll
+    for (int m = i + 1; m < 6; ++m) e -= __shfl_sync(0xffffffffu, L[i], m) * xi[m];
+    xi[i] = e * inv[i];
+  }
+  // the left update: lane 3 i + j holds entry (i, j)
+  const double w0 = xi[3], w1 = xi[4], w2 = xi[5];
+  const double t2 = w0 * w0 + w1 * w1 + w2 * w2;
   const double th = sqrt(t2);
   double a, b, c;
   if (th < 0.05) {  // Maclaurin series of sin t / t, (1 - cos t) / t^2, (t - sin t) / t^3 to t^8 (< 1e-20 left)
@@ -584,91 +727,27 @@ __device__ void se3_left(const double xi[6], double T[kPose]) {
     b = (1.0 - cs) / t2;
     c = (th - sn) / (t2 * th);
   }
-  const double Kx[3][3] = {{0.0, -w[2], w[1]}, {w[2], 0.0, -w[0]}, {-w[1], w[0], 0.0}};
-  double E[3][3], V[3][3];
-  for (int i = 0; i < 3; ++i)
-    for (int j = 0; j < 3; ++j) {
-      const double k2 = Kx[i][0] * Kx[0][j] + Kx[i][1] * Kx[1][j] + Kx[i][2] * Kx[2][j];
-      const double id = i == j ? 1.0 : 0.0;
-      E[i][j] = id + a * Kx[i][j] + b * k2;
-      V[i][j] = id + b * Kx[i][j] + c * k2;
-    }
-  double R[9], t[3];
-  for (int i = 0; i < 3; ++i) {
-    for (int j = 0; j < 3; ++j) R[3 * i + j] = E[i][0] * T[j] + E[i][1] * T[3 + j] + E[i][2] * T[6 + j];
-    t[i] = E[i][0] * T[9] + E[i][1] * T[10] + E[i][2] * T[11] + V[i][0] * xi[0] + V[i][1] * xi[1] + V[i][2] * xi[2];
-  }
-  for (int q = 0; q < 9; ++q) T[q] = R[q];
-  for (int q = 0; q < 3; ++q) T[9 + q] = t[q];
-}
-
-constexpr int kSolveParts = 8;  // partial sums per component in the solve kernel
-
-__global__ void __launch_bounds__(kGnVals * kSolveParts) k_pnp_gn_solve(const double* __restrict__ partials,
-                                                                         State* __restrict__ st) {
-  __shared__ double part[kGnVals][kSolveParts];
-  __shared__ double s[kGnVals];
-  if (!st->active) return;
-  {  // component k, blocks j, j + 8, ... in order; then the 8 parts in order
-    const int k = threadIdx.x / kSolveParts, j = threadIdx.x % kSolveParts;
-    double a = 0.0;
-    for (int b = j; b < kGnBlocks; b += kSolveParts) a += partials[(size_t)b * kGnVals + k];
-    part[k][j] = a;
-  }
-  __syncthreads();
-  if (threadIdx.x < kGnVals) {
-    double a = 0.0;
-    for (int j = 0; j < kSolveParts; ++j) a += part[threadIdx.x][j];
-    s[threadIdx.x] = a;
-  }
-  __syncthreads();
-  if (threadIdx.x != 0) return;
-  if (s[27] < 3.0) {
-    st->active = 0;
-    return;
-  }
-  double H[6][6], L[6][6] = {};
-  int q = 0;
-  for (int r = 0; r < 6; ++r)
-    for (int c = r; c < 6; ++c) {
-      H[r][c] = s[q];
-      H[c][r] = s[q];
-      ++q;
-    }
-  // Cholesky H = L L^T with the reciprocal diagonal: one reciprocal square
-  // root per column and multiplications (fp64 division is a long sequence here)
-  double inv[6];
-  for (int j = 0; j < 6; ++j) {
-    double d = H[j][j];
-    for (int m = 0; m < j; ++m) d -= L[j][m] * L[j][m];
-    if (!(d > 0.0)) {
-      st->active = 0;
-      return;
-    }
-    inv[j] = rsqrt(d);
-    L[j][j] = d * inv[j];
-    for (int i = j + 1; i < 6; ++i) {
-      double e = H[i][j];
-      for (int m = 0; m < j; ++m) e -= L[i][m] * L[j][m];
-      L[i][j] = e * inv[j];
-    }
-  }
-  double y[6], xi[6];
-  for (int i = 0; i < 6; ++i) {  // L y = -g
-    double e = -s[21 + i];
-    for (int m = 0; m < i; ++m) e -= L[i][m] * y[m];
-    y[i] = e * inv[i];
-  }
-  for (int i = 5; i >= 0; --i) {  // L^T xi = y
-    double e = y[i];
-    for (int m = i + 1; m < 6; ++m) e -= L[m][i] * xi[m];
-    xi[i] = e * inv[i];
-  }
-  double T[kPose];
-  for (int p = 0; p < kPose; ++p) T[p] = st->T[p];
-  se3_left(xi, T);
-  for (int p = 0; p < kPose; ++p) st->T[p] = T[p];
-  st->steps += 1;
+  const int i = lane < 9 ? lane / 3 : 2, j = lane < 9 ? lane % 3 : 2;
+  auto kx = [&](int r, int q) -> double {  // [w]x
+    if (r == q) return 0.0;
+    const double v = r + q == 1 ? w2 : r + q == 2 ? w1 : w0;
+    return ((q - r + 3) % 3 == 1) ? -v : v;
+  };
+  const double k2 = kx(i, 0) * kx(0, j) + kx(i, 1) * kx(1, j) + kx(i, 2) * kx(2, j);
+  const double id = i == j ? 1.0 : 0.0, kij = kx(i, j);
+  const double E = id + a * kij + b * k2;
+  const double V = id + b * kij + c * k2;
+  const double e0 = __shfl_sync(0xffffffffu, E, 3 * i), e1 = __shfl_sync(0xffffffffu, E, 3 * i + 1),
+               e2 = __shfl_sync(0xffffffffu, E, 3 * i + 2);
+  const double v0 = __shfl_sync(0xffffffffu, V, 3 * i), v1 = __shfl_sync(0xffffffffu, V, 3 * i + 1),
+               v2 = __shfl_sync(0xffffffffu, V, 3 * i + 2);
+  const double* T = st->T;
+  const double r = e0 * T[j] + e1 * T[3 + j] + e2 * T[6 + j];
+  const double t = e0 * T[9] + e1 * T[10] + e2 * T[11] + v0 * xi[0] + v1 * xi[1] + v2 * xi[2];
+  __syncwarp();  // every lane has read the old pose
+  if (lane < 9) st->T[lane] = r;
+  if (lane < 9 && j == 0) st->T[9 + i] = t;
+  if (lane == 0) st->steps += 1;
 }
 
 // ------------------------------------------------------------------ final inliers
@@ -712,7 +791,9 @@ struct gs_pnp {
   double* X64 = nullptr;
   float4* X32 = nullptr;
   float2* nab = nullptr;
-  float2* pix = nullptr;
+  unsigned* vwords = nullptr;  // validity bits of the matches, whole compaction blocks
+  cudaStream_t side = nullptr;  // P3P, beside the lifting
+  cudaEvent_t ev_scan = nullptr, ev_p3p = nullptr;
   int32_t* vidx = nullptr;
   uint8_t* mask = nullptr;
   double* poses64 = nullptr;
@@ -781,11 +862,14 @@ void gs_pnp_destroy(gs_pnp* s) {
   if (!s) return;
   cudaSetDevice(s->device);
   cudaDeviceSynchronize();
-  for (void* p : {(void*)s->blk, (void*)s->X64, (void*)s->X32, (void*)s->nab, (void*)s->pix, (void*)s->vidx,
+  for (void* p : {(void*)s->blk, (void*)s->X64, (void*)s->X32, (void*)s->nab, (void*)s->vwords, (void*)s->vidx,
                   (void*)s->mask, (void*)s->poses64, (void*)s->poses32, (void*)s->counts, (void*)s->partials,
                   (void*)s->st})
     if (p) cudaFree(p);
   if (s->st_host) cudaFreeHost(s->st_host);
+  if (s->side) cudaStreamDestroy(s->side);
+  if (s->ev_scan) cudaEventDestroy(s->ev_scan);
+  if (s->ev_p3p) cudaEventDestroy(s->ev_p3p);
   for (cudaEvent_t e : s->ev)
     if (e) cudaEventDestroy(e);
   delete s;
@@ -819,7 +903,10 @@ gs_status gs_pnp_create(int64_t max_matches, int max_hypotheses, gs_pnp** out) {
   if ((e = cudaMalloc(&s->X64, 3 * n * sizeof(double))) != cudaSuccess) return bail(e);
   if ((e = cudaMalloc(&s->X32, n * sizeof(float4))) != cudaSuccess) return bail(e);
   if ((e = cudaMalloc(&s->nab, n * sizeof(float2))) != cudaSuccess) return bail(e);
-  if ((e = cudaMalloc(&s->pix, n * sizeof(float2))) != cudaSuccess) return bail(e);
+  if ((e = cudaMalloc(&s->vwords, nb * (kCompact / 32) * sizeof(unsigned))) != cudaSuccess) return bail(e);
+  if ((e = cudaStreamCreateWithFlags(&s->side, cudaStreamNonBlocking)) != cudaSuccess) return bail(e);
+  if ((e = cudaEventCreateWithFlags(&s->ev_scan, cudaEventDisableTiming)) != cudaSuccess) return bail(e);
+  if ((e = cudaEventCreateWithFlags(&s->ev_p3p, cudaEventDisableTiming)) != cudaSuccess) return bail(e);
   if ((e = cudaMalloc(&s->vidx, n * sizeof(int32_t))) != cudaSuccess) return bail(e);
   if ((e = cudaMalloc(&s->mask, n)) != cudaSuccess) return bail(e);
   if ((e = cudaMalloc(&s->poses64, H * kSol * kPose * sizeof(double))) != cudaSuccess) return bail(e);
@@ -876,22 +963,46 @@ gs_status gs_pnp_solve(gs_pnp* s, const gs_camera* cam, const gs_pose* T_render,
   if (n_matches > 0) PNP_CUDA(cudaMemsetAsync(s->mask, 0, (size_t)n_matches, st));
   const int nb = (int)((n_matches + kCompact - 1) / kCompact);
   if (nb > 0) {
-    k_pnp_flags<<<nb, kThreads, 0, st>>>(matches, n_matches, alpha, c.W * c.H, opts->min_alpha, s->blk, s->st);
+    k_pnp_flags<<<nb, kThreads, 0, st>>>(matches, n_matches, alpha, c.W * c.H, opts->min_alpha, s->blk, s->vwords, s->st);
     PNP_CUDA(cudaGetLastError());
   }
   k_pnp_scan<<<1, 1024, 0, st>>>(s->blk, nb, s->st);
   PNP_CUDA(cudaGetLastError());
+  // P3P needs the compaction's counts and bits only and runs beside the lifting
+  // (phase timing keeps them in order)
+  const bool fork = n_hypotheses > 0 && !s->timing;
+  const cudaStream_t ps = fork ? s->side : st;
+  struct Join {  // an error return leaves nothing of this call running beside it
+    cudaStream_t st;
+    bool open;
+    ~Join() {
+      if (open) cudaStreamSynchronize(st);
+    }
+  } join{ps, false};
+  auto p3p = [&]() -> cudaError_t {
+    k_pnp_p3p<<<(n_hypotheses * kSol + 31) / 32, 32, 0, ps>>>(matches, depth, alpha, s->blk, s->vwords, nb, s->st, words,
+                                                              n_hypotheses, c, Tr, s->poses64, s->poses32, s->counts);
+    return cudaGetLastError();
+  };
+  if (fork) {
+    PNP_CUDA(cudaEventRecord(s->ev_scan, st));
+    PNP_CUDA(cudaStreamWaitEvent(ps, s->ev_scan, 0));
+    join.open = true;
+    PNP_CUDA(p3p());
+    PNP_CUDA(cudaEventRecord(s->ev_p3p, ps));
+  }
   if (nb > 0) {
     k_pnp_lift<<<nb, kThreads, 0, st>>>(matches, n_matches, depth, alpha, c, Tr, opts->min_alpha, s->blk, s->X64,
-                                        s->X32, s->nab, s->pix, s->vidx);
+                                        s->X32, s->nab, s->vidx);
     PNP_CUDA(cudaGetLastError());
   }
   PNP_CUDA(mark(1));
   const int n_poses = n_hypotheses * kSol;
-  if (n_hypotheses > 0) {
-    k_pnp_p3p<<<(n_hypotheses + 31) / 32, 32, 0, st>>>(s->X64, s->pix, s->st, words, n_hypotheses, c,
-                                                          s->poses64, s->poses32, s->counts);
-    PNP_CUDA(cudaGetLastError());
+  if (fork) {
+    PNP_CUDA(cudaStreamWaitEvent(st, s->ev_p3p, 0));
+    join.open = false;
+  } else if (n_hypotheses > 0) {
+    PNP_CUDA(p3p());
   }
   PNP_CUDA(mark(2));
   if (n_hypotheses > 0) {
