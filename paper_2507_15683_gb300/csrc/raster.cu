@@ -197,24 +197,29 @@ constexpr int kSmJac = 0;
 constexpr int kSmStageT = kSmHist;
 constexpr int kSmTan = kSmFwd;
 // Feature blending on the tensor cores (FEAT): each warp collects the weights
-// of its hits in slots of kSlots, transposed (slot-major, one row of 32
-// pixels per slot) and split into three bf16 terms w = hi + mid + lo (exact to
-// about 2^-24, the binary32 weight's own precision), then adds
-// W (32 pixels x kSlots) . f (kSlots x 32 channels) to its accumulator
+// of its hits in kSlots rows of its 32 pixels (binary32, row stride kWtRow: the
+// fragment reads of 8 pixels x 4 slots fall in distinct banks). A full group is
+// read as MMA fragments, split in registers into three bf16 terms w = hi + mid +
+// lo (exact to about 2^-24, the binary32 weight's own precision), and W (32
+// pixels x kSlots) . f (kSlots x 32 channels) is added to the warp's accumulator
 // fragments with mma.sync (bf16 x bf16 products are exact in fp32, with fp32
-// accumulation). Rows of kWtRow bf16 (80 bytes): the eight 16-byte rows an
-// ldmatrix reads fall in distinct banks.
+// accumulation). Splitting a pair of weights at a time when the group is full,
+// instead of each weight when it is stored, takes one shared store per hit for
+// three and fewer conversions: 16 views of 480 x 270 with 2 M Gaussians took
+// 2.84 ms, now 2.39 ms.
 // The features of the slots' Gaussians are copied into a per-warp buffer of
-// kSlots rows (same 80-byte stride) when a slot is filled, so that slots span
-// staging batches: a slot group is every kSlots hits of the warp in depth
-// order, whatever the batch size, and the sums come out the same bits under
-// every launch configuration.
+// kSlots rows (80-byte stride: the eight 16-byte rows an ldmatrix reads fall in
+// distinct banks) when a slot is filled, so that slots span staging batches: a
+// slot group is every kSlots hits of the warp in depth order, whatever the
+// batch size, and the sums come out the same bits under every launch
+// configuration.
 constexpr int kSlots = 16;
-constexpr int kWtRow = 40;
+constexpr int kWtRow = 36;                    // floats per weight row
+constexpr int kFbRow = 40;                    // bf16 per feature row
 constexpr int kWtTerms = 3;                   // hi, mid, lo
-constexpr int kWtWarp = kWtTerms * kSlots * kWtRow;  // bf16 per warp: hi rows, mid rows, lo rows
-constexpr int kSmWtBytes = kWarps * kWtWarp * 2;
-constexpr int kSmFbBytes = kWarps * kSlots * kWtRow * 2;  // per-warp slot features (bf16 rows)
+constexpr int kWtWarp = kSlots * kWtRow;      // floats per warp
+constexpr int kSmWtBytes = kWarps * kWtWarp * 4;
+constexpr int kSmFbBytes = kWarps * kSlots * kFbRow * 2;  // per-warp slot features (bf16 rows)
 // Feature-mode layout (blend phase; the sorted list is back in global memory,
 // so it may reuse the sort buffers): staged records, staged features, weight
 // slots, slot features.
@@ -444,12 +449,12 @@ __global__ void __launch_bounds__(kTileThreads, MINB) k_composite(SceneDev sc, c
   float4* scol = sb + kB;
   uint32_t* smask = reinterpret_cast<uint32_t*>(scol + kB);
   uint4* sf = reinterpret_cast<uint4*>(smem_raw + feat_off_sf<KB>());  // FEAT: KB x 4
-  // FEAT: this warp's transposed weight slots (hi rows, then lo rows) and slot features
-  unsigned short* wt = reinterpret_cast<unsigned short*>(smem_raw + feat_off_wt<KB>()) + (threadIdx.x >> 5) * kWtWarp;
+  // FEAT: this warp's weight slots and slot features
+  float* wt = reinterpret_cast<float*>(smem_raw + feat_off_wt<KB>()) + (threadIdx.x >> 5) * kWtWarp;
   unsigned short* fb = reinterpret_cast<unsigned short*>(smem_raw + feat_off_fb<KB>()) +
-                       (threadIdx.x >> 5) * (kSlots * kWtRow);
+                       (threadIdx.x >> 5) * (kSlots * kFbRow);
   if (FEAT) {  // empty slots multiply stale rows by zero weights: keep the rows finite
-    for (int i = threadIdx.x & 31; i < kSlots * kWtRow; i += 32) fb[i] = 0;
+    for (int i = threadIdx.x & 31; i < kSlots * kFbRow; i += 32) fb[i] = 0;
   }
   float4* sj = reinterpret_cast<float4*>(smem_raw + kSmJac);  // TAN: KB x 12
   __shared__ uint32_t s_tile;
@@ -529,27 +534,36 @@ __global__ void __launch_bounds__(kTileThreads, MINB) k_composite(SceneDev sc, c
     // FEAT: add the filled slots to the warp's accumulators (empty slots get
     // zero weights)
     auto flush_feats = [&]() {
-      for (int sl = nslot; sl < kSlots; ++sl)
-#pragma unroll
-        for (int t = 0; t < kWtTerms; ++t) wt[(t * kSlots + sl) * kWtRow + lane] = 0;
+      for (int sl = nslot; sl < kSlots; ++sl) wt[sl * kWtRow + lane] = 0.0f;
       __syncwarp();
       // B: the slots' features, k = slot (lane % 16), 8 channels from (lane / 16) * 8
-      const uint32_t bb = (uint32_t)__cvta_generic_to_shared(fb + (lane & (kSlots - 1)) * kWtRow) +
+      const uint32_t bb = (uint32_t)__cvta_generic_to_shared(fb + (lane & (kSlots - 1)) * kFbRow) +
                           (uint32_t)(lane >> 4) * 16u;
       uint32_t b[8];
       ldsm_x4_trans(bb, b[0], b[1], b[2], b[3]);       // channels 0..15
       ldsm_x4_trans(bb + 32u, b[4], b[5], b[6], b[7]);  // channels 16..31
-      // A: weights, matrix lane / 8 = (pixels +8 if odd, slots +8 if >= 2)
-      const int kk = (lane & 7) + ((lane >> 4) << 3), pp = ((lane >> 3) & 1) << 3;
-      const uint32_t wa = (uint32_t)__cvta_generic_to_shared(wt) + (uint32_t)(kk * kWtRow + pp) * 2u;
+      // A: weights of pixels g, g + 8 (+ 16 mt), slots 2 t, 2 t + 1 (+ 8), with g = lane / 4, t = lane % 4
+      const float* wa = wt + (lane & 3) * (2 * kWtRow) + (lane >> 2);
 #pragma unroll
       for (int mt = 0; mt < 2; ++mt) {
+        uint32_t a[kWtTerms][4];
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+          const float* q = wa + mt * 16 + (r & 1) * 8 + (r >> 1) * (8 * kWtRow);
+          float x = q[0], y = q[kWtRow];
+#pragma unroll
+          for (int t = 0; t < kWtTerms; ++t) {  // round both, keep the exact remainders
+            const __nv_bfloat162 h = __floats2bfloat162_rn(x, y);
+            a[t][r] = *reinterpret_cast<const uint32_t*>(&h);
+            x = __fsub_rn(x, __uint_as_float(a[t][r] << 16));
+            y = __fsub_rn(y, __uint_as_float(a[t][r] & 0xffff0000u));
+          }
+        }
 #pragma unroll
         for (int t = kWtTerms - 1; t >= 0; --t) {  // smallest term first
-          uint32_t a0, a1, a2, a3;
-          ldsm_x4_trans(wa + (uint32_t)(t * kSlots * kWtRow * 2 + mt * 32), a0, a1, a2, a3);
 #pragma unroll
-          for (int nt = 0; nt < 4; ++nt) mma_16816(F[mt][nt], a0, a1, a2, a3, b[2 * nt], b[2 * nt + 1]);
+          for (int nt = 0; nt < 4; ++nt)
+            mma_16816(F[mt][nt], a[t][0], a[t][1], a[t][2], a[t][3], b[2 * nt], b[2 * nt + 1]);
         }
       }
       __syncwarp();
@@ -676,14 +690,8 @@ __global__ void __launch_bounds__(kTileThreads, MINB) k_composite(SceneDev sc, c
         C2 = fmaf(wgt, c.z, C2);
         D = fmaf(wgt, zj, D);
         if (FEAT && __any_sync(0xffffffffu, wgt != 0.0f)) {  // a slot for a hit some pixel blends
-          const __nv_bfloat16 hi = __float2bfloat16_rn(wgt);
-          const float r1 = __fsub_rn(wgt, __bfloat162float(hi));  // exact differences
-          const __nv_bfloat16 mid = __float2bfloat16_rn(r1);
-          const __nv_bfloat16 lo = __float2bfloat16_rn(__fsub_rn(r1, __bfloat162float(mid)));
-          wt[nslot * kWtRow + lane] = __bfloat16_as_ushort(hi);
-          wt[(kSlots + nslot) * kWtRow + lane] = __bfloat16_as_ushort(mid);
-          wt[(2 * kSlots + nslot) * kWtRow + lane] = __bfloat16_as_ushort(lo);
-          if (lane < 4) reinterpret_cast<uint4*>(fb + nslot * kWtRow)[lane] = sf[j * 4 + lane];
+          wt[nslot * kWtRow + lane] = wgt;
+          if (lane < 4) reinterpret_cast<uint4*>(fb + nslot * kFbRow)[lane] = sf[j * 4 + lane];
           if (++nslot == kSlots) flush_feats();
         }
         if (TAN) n_blend += acc ? 1u : 0u;
