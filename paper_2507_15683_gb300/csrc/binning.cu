@@ -27,11 +27,17 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_tiles(Work w) {
   const uint32_t n = w.n_tiles;
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   if (tid == 0) s_carry = 0ull;
+  pdl_wait();
   for (uint32_t base = 0; base < n; base += kScanChunk) {  // block-uniform
 #pragma unroll
     for (int i = 0; i < kScanPer; ++i) {
       const uint32_t k = base + (uint32_t)(i * kScanThreads + tid);
       sv[i * kScanThreads + tid] = k < n ? w.tile_count[k] : 0u;
+    }
+#pragma unroll
+    for (int i = 0; i < kScanPer; ++i) {  // the next call counts from zero
+      const uint32_t k = base + (uint32_t)(i * kScanThreads + tid);
+      if (k < n) w.tile_count[k] = 0u;
     }
     __syncthreads();
     // this thread's kScanPer consecutive counts, as two 16-byte reads
@@ -91,6 +97,7 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_tiles(Work w) {
     }
     __syncthreads();  // sv and s_carry are reused by the next chunk
   }
+  pdl_trigger();
   // the view counters of the tangent pass's chunked reduction start at zero every call
   for (uint32_t k = tid; k < w.n_views && w.n_chunks; k += kScanThreads) w.view_ctr[k] = 0u;
   if (tid == 0) {
@@ -113,6 +120,8 @@ constexpr int kScatterUnroll = 8;
 __global__ void __launch_bounds__(256) k_scatter(const View* __restrict__ views, Work w) {
   __shared__ uint32_t s_incl[8][32];
   __shared__ uint4 s_m[8][32];
+  pdl_wait();
+  pdl_trigger();
   if (w.ctr->overflow) return;
   // every slot a tile cursor hands out lies below the scanned total when the
   // projection's tile counts and the records' rectangles agree; a slot past it
@@ -313,6 +322,7 @@ __device__ void warp_sort_list(uint2* __restrict__ list, int n, const float4* __
 
 __global__ void __launch_bounds__(256, 4) k_sort_tiles(Work w) {
   __shared__ uint32_t s_rec[8][kWarpSortMax];
+  pdl_wait();
   if (w.ctr->overflow) return;
   const int lane = threadIdx.x & 31;
   uint32_t* srec = s_rec[threadIdx.x >> 5];
@@ -331,19 +341,16 @@ __global__ void __launch_bounds__(256, 4) k_sort_tiles(Work w) {
 
 }  // namespace
 
-cudaError_t launch_sort_tiles(const Work& w, int grid, cudaStream_t st) {
-  k_sort_tiles<<<grid, 256, 0, st>>>(w);
-  return cudaGetLastError();
+cudaError_t launch_sort_tiles(const Work& w, int grid, cudaStream_t st, bool early) {
+  return launch_dependent(early, k_sort_tiles, grid, 256, st, w);
 }
 
-cudaError_t launch_scan_tiles(const Work& w, cudaStream_t st) {
-  k_scan_tiles<<<1, kScanThreads, 0, st>>>(w);
-  return cudaGetLastError();
+cudaError_t launch_scan_tiles(const Work& w, cudaStream_t st, bool early) {
+  return launch_dependent(early, k_scan_tiles, 1, kScanThreads, st, w);
 }
 
-cudaError_t launch_scatter(const View* views, const Work& w, int grid, cudaStream_t st) {
-  k_scatter<<<grid, 256, 0, st>>>(views, w);
-  return cudaGetLastError();
+cudaError_t launch_scatter(const View* views, const Work& w, int grid, cudaStream_t st, bool early) {
+  return launch_dependent(early, k_scatter, grid, 256, st, views, w);
 }
 
 }  // namespace gsr

@@ -174,7 +174,8 @@ struct gs_scene {
   uint32_t tile_cap = 0;
   DevBuf pairs, pairs_tmp;
   uint32_t pair_cap = 0;
-  DevBuf ctr, result, views;
+  DevBuf result, views;     // views: the call table (counters, index ranges, views)
+  bool counts_zero = false;  // tile_count is all zeros (the scan leaves it so)
   Counters* ctr_host = nullptr;
   double* result_host = nullptr;
   // loss targets uploaded from host memory (gs_render_pose_grad_host) on a side
@@ -275,7 +276,7 @@ Work work_of(gs_scene* s, uint32_t n_tiles) {
   w.pairs = dp<uint2>(s->pairs);
   w.pairs_tmp = dp<uint2>(s->pairs_tmp);
   w.pair_cap = s->pair_cap;
-  w.ctr = dp<Counters>(s->ctr);
+  w.ctr = dp<Counters>(s->views);
   w.partials = dp<double>(s->partials);
   // chunk sums, then the view counters; one view has at least one tile, so
   // tile_cap bounds both the chunk and the view count
@@ -317,6 +318,7 @@ gs_status grow_pairs(gs_scene* s, uint64_t pair_cap) {
 gs_status grow_tiles(gs_scene* s, uint64_t n_tiles) {
   if (n_tiles + 1 > s->tile_cap) {
     const uint64_t cap = n_tiles + 1;
+    s->counts_zero = false;
     GS_TRY(ensure(s->tile_count, cap * sizeof(uint32_t)));
     GS_TRY(ensure(s->tile_offset, cap * sizeof(uint32_t)));
     GS_TRY(ensure(s->tile_cursor, cap * sizeof(uint32_t)));
@@ -410,13 +412,24 @@ gs_status build_views(gs_scene* s, int nv, const gs_camera* cams, const gs_pose*
 // it (pinned memory, for graph capture); otherwise from hv (pageable: the copy
 // is staged before cudaMemcpyAsync returns).
 // Device call table: ranges (1 + partitions entries) followed by the views.
-size_t table_ranges_bytes(const gs_scene* s) { return (1 + s->parts.size()) * sizeof(int4); }
-size_t table_bytes(const gs_scene* s, int nv) { return table_ranges_bytes(s) + (size_t)nv * sizeof(View); }
+// In front of both stand the call's counters: the table's upload zeroes them.
+constexpr size_t kCtrBytes = (sizeof(Counters) + 255) / 256 * 256;
+size_t table_views_off(const gs_scene* s) { return kCtrBytes + (1 + s->parts.size()) * sizeof(int4); }
+size_t table_bytes(const gs_scene* s, int nv) { return table_views_off(s) + (size_t)nv * sizeof(View); }
 
 void fill_table(const gs_scene* s, const std::vector<View>& hv, const std::vector<int4>& ranges, char* dst) {
-  std::memset(dst, 0, table_ranges_bytes(s));
-  std::memcpy(dst, ranges.data(), ranges.size() * sizeof(int4));
-  std::memcpy(dst + table_ranges_bytes(s), hv.data(), hv.size() * sizeof(View));
+  std::memset(dst, 0, table_views_off(s));
+  std::memcpy(dst + kCtrBytes, ranges.data(), ranges.size() * sizeof(int4));
+  std::memcpy(dst + table_views_off(s), hv.data(), hv.size() * sizeof(View));
+}
+
+// The per-tile counts start at zero: the scan leaves them so, and they are only
+// cleared here when they are new or a call failed between the two.
+gs_status zero_counts(gs_scene* s, cudaStream_t st) {
+  if (s->counts_zero) return GS_OK;
+  GS_CUDA(cudaMemsetAsync(s->tile_count.p, 0, (size_t)s->tile_cap * sizeof(uint32_t), st));
+  s->counts_zero = true;
+  return GS_OK;
 }
 
 // `graph`: the call is being captured (no timing events). `after_table`, if
@@ -443,9 +456,10 @@ gs_status enqueue(gs_scene* s, const std::vector<View>& hv, const std::vector<in
     GS_TRY(ensure(s->vis_acc, (size_t)s->rec_cap * kVisAcc * sizeof(float)));
     GS_TRY(ensure(s->vis_blk, ((size_t)s->n / kVisBlock + 1) * sizeof(uint32_t)));
   }
-  View* dviews = reinterpret_cast<View*>(static_cast<char*>(s->views.p) + table_ranges_bytes(s));
+  View* dviews = reinterpret_cast<View*>(static_cast<char*>(s->views.p) + table_views_off(s));
   if (keep_table) {
     // the device table is current (a device-side pose update rewrote it)
+    GS_CUDA(cudaMemsetAsync(s->views.p, 0, sizeof(Counters), st));
   } else if (upload_src) {
     GS_CUDA(cudaMemcpyAsync(s->views.p, upload_src, table_bytes(s, nv), cudaMemcpyHostToDevice, st));
   } else {
@@ -455,14 +469,13 @@ gs_status enqueue(gs_scene* s, const std::vector<View>& hv, const std::vector<in
   }
   if (after_table) GS_TRY((*after_table)());
   Work w = work_of(s, (uint32_t)n_tiles);
-  w.ranges = dp<int4>(s->views);
+  w.ranges = reinterpret_cast<const int4*>(static_cast<const char*>(s->views.p) + kCtrBytes);
   if (g) {
     const View& L = hv.back();
     w.n_chunks = L.chunk_base + (uint32_t)(((uint64_t)L.tiles_x * L.tiles_y + kChunkTiles - 1) / kChunkTiles);
     w.n_views = (uint32_t)nv;
   }
-  GS_CUDA(cudaMemsetAsync(w.tile_count, 0, (n_tiles + 1) * sizeof(uint32_t), st));
-  GS_CUDA(cudaMemsetAsync(w.ctr, 0, sizeof(Counters), st));
+  if (!graph) GS_TRY(zero_counts(s, st));  // a captured call: before its launch
   const SceneDev sc = scene_dev(s);
   std::vector<cudaEvent_t> ev;
   const bool timed = s->timing && !graph;  // no events inside captured graphs
@@ -482,6 +495,7 @@ gs_status enqueue(gs_scene* s, const std::vector<View>& hv, const std::vector<in
   const int mode = g ? kModeTan : (feats && s->feat_dim) ? kModeFwdFeat : kModeFwd;
   const int grid = s->sm_count * std::max(1, cfg.grid_mult[mode]);  // projection, shading, scatter, sort
   GS_CUDA(mark(0));
+  if (!graph) s->counts_zero = false;  // until the scan is on the stream
   GS_CUDA(launch_project(sc, dviews, nv, w, grid, st));
   GS_CUDA(mark(1));
   // The shading pass reads only what the projection wrote, and the binning
@@ -503,11 +517,16 @@ gs_status enqueue(gs_scene* s, const std::vector<View>& hv, const std::vector<in
     GS_CUDA(launch_shade(sc, dviews, w, jac, grid, st));
   }
   GS_CUDA(mark(2));
-  GS_CUDA(launch_scan_tiles(w, st));
+  // Early starts of the binning pay where the shading beside it is short: the
+  // 1080p render took 264 us without them, 254 us with them; with the pose
+  // Jacobian the waiting blocks hold registers that the shading needs (gradient
+  // 634 -> 648 us, visibility check 680 -> 703 us).
+  GS_CUDA(launch_scan_tiles(w, st, !jac));
+  if (!graph) s->counts_zero = true;
   GS_CUDA(mark(3));
-  GS_CUDA(launch_scatter(dviews, w, grid, st));
+  GS_CUDA(launch_scatter(dviews, w, grid, st, !jac));
   GS_CUDA(mark(4));
-  GS_CUDA(launch_sort_tiles(w, grid, st));
+  GS_CUDA(launch_sort_tiles(w, grid, st, !jac));
   if (fork) GS_CUDA(cudaStreamWaitEvent(st, s->ev_shade, 0));
   GS_CUDA(mark(5));
   if (!g || feats) GS_CUDA(launch_composite(sc, dviews, nv, w, feats, cfg, s->sm_count, st));
@@ -693,7 +712,7 @@ std::vector<uint32_t> filled_records(const Counters& c, uint32_t rec_cap) {
 }
 
 gs_status read_counters(gs_scene* s, cudaStream_t st, Counters& c) {
-  GS_CUDA(cudaMemcpyAsync(s->ctr_host, s->ctr.p, sizeof(Counters), cudaMemcpyDeviceToHost, st));
+  GS_CUDA(cudaMemcpyAsync(s->ctr_host, s->views.p, sizeof(Counters), cudaMemcpyDeviceToHost, st));
   GS_CUDA(cudaStreamSynchronize(st));
   c = *s->ctr_host;
   return GS_OK;
@@ -721,7 +740,7 @@ gs_status run_sync(gs_scene* s, const std::vector<View>& hv, uint64_t n_tiles, c
   for (int attempt = 0; attempt < 4; ++attempt) {
     GS_TRY(enqueue(s, hv, ranges, n_tiles, g, st, s->table_host, targets_ready, vis, bands, false,
                    attempt == 0 ? after_table : nullptr));
-    GS_CUDA(cudaMemcpyAsync(s->ctr_host, s->ctr.p, sizeof(Counters), cudaMemcpyDeviceToHost, st));
+    GS_CUDA(cudaMemcpyAsync(s->ctr_host, s->views.p, sizeof(Counters), cudaMemcpyDeviceToHost, st));
     if (g && !g->result)
       GS_CUDA(cudaMemcpyAsync(s->result_host, s->result.p, 7 * sizeof(double), cudaMemcpyDeviceToHost, st));
     GS_CUDA(cudaStreamSynchronize(st));
@@ -808,12 +827,13 @@ gs_status run_graph(gs_scene* s, GraphCache& G, const std::vector<char>& key, co
     // capture on a private stream (the legacy default stream cannot be captured);
     // the graph is then launched on the caller's stream
     if (!G.capture) GS_CUDA(cudaStreamCreateWithFlags(&G.capture, cudaStreamNonBlocking));
+    GS_TRY(zero_counts(s, st));
     GS_CUDA(cudaStreamSynchronize(st));
     cudaGraph_t graph = nullptr;
     GS_CUDA(cudaStreamBeginCapture(G.capture, cudaStreamCaptureModeThreadLocal));
     gs_status est = enqueue(s, hv, ranges, n_tiles, g, G.capture, G.host_table, nullptr, nullptr, nullptr, true);
     if (est == GS_OK && copy_back) {  // the counters and the (loss, gradient) to the pinned host copies
-      if (cudaMemcpyAsync(s->ctr_host, s->ctr.p, sizeof(Counters), cudaMemcpyDeviceToHost, G.capture) != cudaSuccess ||
+      if (cudaMemcpyAsync(s->ctr_host, s->views.p, sizeof(Counters), cudaMemcpyDeviceToHost, G.capture) != cudaSuccess ||
           (g && cudaMemcpyAsync(s->result_host, s->result.p, 7 * sizeof(double), cudaMemcpyDeviceToHost, G.capture) !=
                     cudaSuccess))
         est = fail(GS_ERR_CUDA, "cudaMemcpyAsync in the captured call failed");
@@ -836,6 +856,7 @@ gs_status run_graph(gs_scene* s, GraphCache& G, const std::vector<char>& key, co
     s->last_views = hv;
     s->last_tiles = (uint32_t)n_tiles;
   }
+  GS_TRY(zero_counts(s, st));
   GS_CUDA(cudaGraphLaunch(G.exec, st));
   GS_CUDA(cudaEventRecord(G.done, st));
   return GS_OK;
@@ -946,7 +967,6 @@ gs_status gs_create_scene(const gs_scene_desc* d, gs_scene** out) {
   if ((st = ensure(s->cov, 2 * n * sizeof(float4))) != GS_OK) return cleanup(st);
   if ((st = ensure(s->sh, n * s->nsh4 * sizeof(float4))) != GS_OK) return cleanup(st);
   if (s->feat_dim && (st = ensure(s->feat, n * 4 * sizeof(uint4))) != GS_OK) return cleanup(st);
-  if ((st = ensure(s->ctr, sizeof(Counters))) != GS_OK) return cleanup(st);
   if ((st = ensure(s->result, 8 * sizeof(double))) != GS_OK) return cleanup(st);
   if (cudaMallocHost(&s->ctr_host, sizeof(Counters)) != cudaSuccess ||
       cudaMallocHost(&s->result_host, 8 * sizeof(double)) != cudaSuccess) {
@@ -995,6 +1015,9 @@ gs_status gs_create_scene(const gs_scene_desc* d, gs_scene** out) {
       s->parts.push_back(P);
     }
   }
+  if ((st = ensure(s->views, table_bytes(s, 1))) != GS_OK) return cleanup(st);
+  if ((e = cudaMemset(s->views.p, 0, kCtrBytes)) != cudaSuccess)
+    return cleanup(fail(GS_ERR_CUDA, std::string("cudaMemset: ") + cudaGetErrorString(e)));
   s->streaming = !d->device_resident && d->n_partitions > 0 && n > 0;
   if (s->streaming) {
     // pack on the host into pinned memory in the device layout; partitions are
@@ -1080,7 +1103,7 @@ void gs_destroy_scene(gs_scene* s) {
     for (cudaEvent_t e : ev) cudaEventDestroy(e);
   for (DevBuf* b : {&s->pos, &s->cov, &s->sh, &s->feat, &s->rec_a, &s->rec_b, &s->rec_c, &s->rec_m, &s->rec_j,
                     &s->tile_count, &s->tile_offset, &s->tile_cursor, &s->partials, &s->chunks, &s->pairs, &s->pairs_tmp,
-                    &s->ctr, &s->result, &s->views, &s->vis_T, &s->vis_last, &s->vis_acc, &s->vis_uv, &s->vis_blk})
+                    &s->result, &s->views, &s->vis_T, &s->vis_last, &s->vis_acc, &s->vis_uv, &s->vis_blk})
     release(*b);
   for (void* h : {(void*)s->h_pos, (void*)s->h_cov, (void*)s->h_sh, (void*)s->h_feat})
     if (h) cudaFreeHost(h);
@@ -1837,6 +1860,7 @@ __global__ void __launch_bounds__(128) k_refine_update(View* __restrict__ views,
                                                        unsigned int* __restrict__ sticky) {
   const int v = blockIdx.x * 4 + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
+  pdl_wait();
   if (v >= nv) return;
   const unsigned int bad = ctr->overflow | (ctr->error ? 0x100u : 0u);
   if (bad) {  // this iteration's render is incomplete: stop updating
@@ -1972,10 +1996,9 @@ gs_status refine_on_device(gs_scene* s, int nv, const gs_camera* cams, gs_pose* 
   const int blocks = (nv + 3) / 4;
   gs_status status = GS_OK;
   auto launch_update = [&](cudaStream_t on) -> gs_status {
-    View* dviews = reinterpret_cast<View*>(static_cast<char*>(s->views.p) + table_ranges_bytes(s));
-    k_refine_update<<<blocks, 128, 0, on>>>(dviews, nv, dp<double>(s->result), drs, *o, iters, dhist,
-                                            dp<Counters>(s->ctr), dsticky);
-    GS_CUDA(cudaGetLastError());
+    View* dviews = reinterpret_cast<View*>(static_cast<char*>(s->views.p) + table_views_off(s));
+    GS_CUDA(launch_dependent(true, k_refine_update, blocks, 128, on, dviews, nv, dp<double>(s->result), drs, *o, iters, dhist,
+                             dp<Counters>(s->views), dsticky));
     return GS_OK;
   };
   for (int attempt = 0;; ++attempt) {

@@ -89,7 +89,7 @@ struct Work {
   float* rec_j;        // kJacStride floats per record (pose gradient only)
   uint32_t rec_cap;    // multiple of kRecRegions
   uint32_t rec_seg;    // rec_cap / kRecRegions
-  uint32_t* tile_count;   // n_tiles + 1
+  uint32_t* tile_count;   // n_tiles + 1; zero before the projection, and again after the scan
   uint32_t* tile_offset;  // n_tiles + 1 (exclusive scan)
   uint32_t* tile_cursor;  // n_tiles
   uint32_t n_tiles;
@@ -133,6 +133,29 @@ struct LaunchCfg {
   int grid_mult[kModeCount] = {8, 8, 8};
 };
 
+// A kernel launched by launch_dependent may start (its blocks become resident)
+// before the kernel in front of it on the stream has ended, once all blocks of
+// that one have called pdl_trigger or exited; it calls pdl_wait before anything
+// else, which returns when that kernel has completed. So the launch and the
+// block scheduling of one kernel of a chain hide behind the last blocks of the
+// kernel before. Without `early` it is an ordinary launch. Every kernel launched this way waits on every path, so the
+// completion of one implies that of all kernels before it.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+template <typename... P, typename... A>
+cudaError_t launch_dependent(bool early, void (*kernel)(P...), int grid, int block, cudaStream_t st, A... args) {
+  cudaLaunchAttribute attr;
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = early ? 1 : 0;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)grid);
+  cfg.blockDim = dim3((unsigned)block);
+  cfg.stream = st;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
+
 // launchers (return the CUDA error of the launch)
 cudaError_t launch_pack_scene(const float* means, const float* scales, const float* quats,
                               const float* opacities, const float* sh, int sh_k3, const uint16_t* feats,
@@ -142,9 +165,9 @@ cudaError_t launch_project(const SceneDev& sc, const View* views, int n_views, c
                            cudaStream_t st);
 cudaError_t launch_shade(const SceneDev& sc, const View* views, const Work& w, bool grad, int grid,
                          cudaStream_t st);
-cudaError_t launch_scan_tiles(const Work& w, cudaStream_t st);
-cudaError_t launch_sort_tiles(const Work& w, int grid, cudaStream_t st);
-cudaError_t launch_scatter(const View* views, const Work& w, int grid, cudaStream_t st);
+cudaError_t launch_scan_tiles(const Work& w, cudaStream_t st, bool early = false);
+cudaError_t launch_sort_tiles(const Work& w, int grid, cudaStream_t st, bool early = false);
+cudaError_t launch_scatter(const View* views, const Work& w, int grid, cudaStream_t st, bool early = false);
 // feats: some view writes the feature map (else the feature-free kernel runs);
 // persistent grid from cfg and the SM count
 cudaError_t launch_composite(const SceneDev& sc, const View* views, int n_views, const Work& w, bool feats,

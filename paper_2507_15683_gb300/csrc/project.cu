@@ -332,6 +332,7 @@ __global__ void __launch_bounds__(256) k_project(SceneDev sc, const View* __rest
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const unsigned lt_mask = (1u << lane) - 1u;
   const unsigned region = blockIdx.x % kRecRegions;
+  pdl_trigger();
   const int4 hdr = w.ranges[0];  // (ranges, total length): only partitions in view are walked
   int2* q = s_q[wid];
   float4* qp = s_qp[wid];

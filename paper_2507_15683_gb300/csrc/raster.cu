@@ -369,6 +369,8 @@ __device__ void tile_partial(float (&v)[7], uint32_t tile, int tid, int lane, in
 __global__ void __launch_bounds__(7 * 32) k_reduce_chunks(const View* __restrict__ views, int n_views, Work w,
                                                           double* __restrict__ result) {
   __shared__ bool s_last;
+  pdl_wait();
+  pdl_trigger();
   if (w.ctr->overflow) return;
   const uint32_t chunk = blockIdx.x;
   const int lane = threadIdx.x & 31, k = threadIdx.x >> 5;
@@ -461,6 +463,7 @@ __global__ void __launch_bounds__(kTileThreads, MINB) k_composite(SceneDev sc, c
   __shared__ uint32_t s_tmp[kWarps];
   __shared__ float s_red[kWarps][8];
   (void)result;  // the tangent pass's fp64 sums are k_reduce_chunks's
+  if (TAN) pdl_trigger();
   if (w.ctr->overflow) return;
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   int lx, ly, bxw, byw;
@@ -1034,8 +1037,7 @@ cudaError_t launch_composite_tangent(const SceneDev& sc, const View* views, int 
 
 cudaError_t launch_reduce_tangent(const View* views, int n_views, const Work& w, double* result, cudaStream_t st) {
   if (w.n_tiles == 0 || w.n_chunks == 0) return cudaSuccess;
-  k_reduce_chunks<<<w.n_chunks, 7 * 32, 0, st>>>(views, n_views, w, result);
-  return cudaGetLastError();
+  return launch_dependent(true, k_reduce_chunks, (int)w.n_chunks, 7 * 32, st, views, n_views, w, result);
 }
 
 cudaError_t launch_composite_tangent_range(const SceneDev& sc, const View* views, int n_views, const Work& w,
