@@ -288,6 +288,13 @@ gs_status gs_scene_stream_stats(gs_scene* scene, int64_t* h2d_bytes, int* reside
                                 int* active_partitions);
 gs_status gs_scene_evict(gs_scene* scene);
 
+/* Copy n device arrays to n others, all in one launch (the result arrays of a
+ * matcher or solver, which belong to it, into a caller's own): bytes[i] bytes
+ * from src[i] to dst[i], which must not overlap; empty arrays may be NULL.
+ * Asynchronous on `stream`. Errors: INVALID_ARG (n outside [0, 16], a negative
+ * size, a NULL array of a positive size), CUDA. */
+gs_status gs_copy_arrays(int n, void* const* dst, const void* const* src, const int64_t* bytes, void* stream);
+
 /* Gaussian count, SH degree and feature channels of a scene (host pointers,
  * each may be NULL). Errors: INVALID_ARG (NULL scene). */
 gs_status gs_scene_shape(const gs_scene* scene, int64_t* n, int* sh_degree, int* feat_dim);

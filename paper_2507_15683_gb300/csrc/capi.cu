@@ -1364,6 +1364,26 @@ gs_status gs_scene_stream_stats(gs_scene* s, int64_t* h2d_bytes, int* resident_p
   return GS_OK;
 }
 
+gs_status gs_copy_arrays(int n, void* const* dst, const void* const* src, const int64_t* bytes, void* stream) {
+  g_err.clear();
+  if (n < 0 || n > kCopyMax) return fail(GS_ERR_INVALID_ARG, "gs_copy_arrays takes 0 to 16 arrays");
+  if (n > 0 && (!dst || !src || !bytes)) return fail(GS_ERR_INVALID_ARG, "dst, src and bytes are required");
+  CopyList c;
+  for (int i = 0; i < n; ++i) {
+    if (bytes[i] < 0 || (bytes[i] > 0 && (!dst[i] || !src[i])))
+      return fail(GS_ERR_INVALID_ARG, "a negative size or a NULL array");
+    if (bytes[i] == 0) continue;
+    c.dst[c.n] = static_cast<char*>(dst[i]);
+    c.src[c.n] = static_cast<const char*>(src[i]);
+    c.bytes[c.n++] = bytes[i];
+  }
+  int dev = 0, sms = 1;
+  GS_CUDA(cudaGetDevice(&dev));
+  GS_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+  GS_CUDA(launch_copy(c, sms, (cudaStream_t)stream));
+  return GS_OK;
+}
+
 gs_status gs_scene_shape(const gs_scene* s, int64_t* n, int* sh_degree, int* feat_dim) {
   g_err.clear();
   GS_TRY(check_scene(s));

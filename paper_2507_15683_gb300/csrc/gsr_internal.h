@@ -197,6 +197,16 @@ cudaError_t launch_vis_inimage(const SceneDev& sc, const View* views, uint8_t* m
 // every record: mean gradient of sum RGB, M^r (bit 1), M (bit 0), count
 cudaError_t launch_vis_chain(const View* views, const Work& w, const float* acc, uint8_t* mask, float* grad,
                              int grid, cudaStream_t st);
+// device arrays copied in one launch, at most kCopyMax
+constexpr int kCopyMax = 16;
+struct CopyList {
+  int n = 0;
+  char* dst[kCopyMax];
+  const char* src[kCopyMax];
+  long long bytes[kCopyMax];
+};
+cudaError_t launch_copy(const CopyList& c, int sm_count, cudaStream_t st);
+
 // kept Gaussians in ascending order: ids and (U, V); blk holds n / kVisBlock + 1 counters
 cudaError_t launch_vis_compact(const uint8_t* mask, const float2* uv, int n, uint32_t* blk, int32_t* vis_gid,
                                float2* vis_uv, cudaStream_t st);

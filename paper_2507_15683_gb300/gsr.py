@@ -150,6 +150,7 @@ def _load():
         "gs_dense_localize": [vp, vp, vp, P(gs_camera), P(gs_pose), vp, vp, P(gs_localize_opts),
                               P(gs_localize_result), vp],
         "gs_scene_shape": [vp, vp, vp, vp],
+        "gs_copy_arrays": [st, vp, vp, vp, vp],
         "gs_pmm_shape": [vp, vp, vp, vp],
         "gs_pmm_set_wait_limit": [vp, st],
         "gs_scene_set_launch": [vp, st, st, P(gs_camera), P(gs_launch)],
@@ -676,12 +677,23 @@ def gs_pmm_match(h, feat_query: int, feat_render: int, tau: float, stream: int) 
     return r
 
 
-class _DevView:
-    """A device array of the library, seen by torch without a copy."""
+def gs_copy_arrays(dst, src, nbytes, stream: int) -> None:
+    """Device arrays (addresses, sizes in bytes) copied in one launch."""
+    n = len(dst)
+    vp = ctypes.c_void_p * n
+    _check(lib.gs_copy_arrays(n, vp(*dst), vp(*src), (ctypes.c_int64 * n)(*nbytes), stream))
 
-    def __init__(self, ptr: int, shape, typestr: str):
-        self.__cuda_array_interface__ = {"shape": tuple(int(x) for x in shape), "typestr": typestr,
-                                         "data": (int(ptr or 0), False), "version": 3, "strides": None}
+
+def _copied(arrays: dict) -> dict:
+    """Tensors of their own with the contents of the library's device arrays:
+    {name: (address, shape, torch dtype)}. (Wrapping each array as a tensor and
+    cloning it took about 15 us of host time apiece and a launch each.)"""
+    import torch
+    out = {k: torch.empty(shape, dtype=dt, device="cuda") for k, (_, shape, dt) in arrays.items()}
+    ts = list(out.values())
+    gs_copy_arrays([t.data_ptr() for t in ts], [a[0] for a in arrays.values()],
+                   [t.numel() * t.element_size() for t in ts], _stream())
+    return out
 
 
 class Matcher:
@@ -716,14 +728,12 @@ class Matcher:
         import torch
         r = self.match_raw(feat_query, feat_render, tau)
         n, nc, nf = r.n_cells, r.n_coarse, r.n_fine
-        v = lambda p, shape, t: torch.as_tensor(_DevView(p, shape, t), device="cuda").clone()
-        return {"codes_q": v(r.codes_q, (n, 64), "<u2"), "codes_r": v(r.codes_r, (n, 64), "<u2"),
-                "lse_row": v(r.lse_row, (n,), "<f4"), "lse_col": v(r.lse_col, (n,), "<f4"),
-                "row_best": v(r.row_best, (n,), "<i4"), "col_best": v(r.col_best, (n,), "<i4"),
-                "coarse": v(r.coarse, (nc, 2), "<i4") if nc else torch.zeros((0, 2), dtype=torch.int32, device="cuda"),
-                "coarse_prob": v(r.coarse_prob, (nc,), "<f4") if nc else torch.zeros(0, device="cuda"),
-                "fine": v(r.fine, (nf, 3), "<i4") if nf else torch.zeros((0, 3), dtype=torch.int32, device="cuda"),
-                "fine_prob": v(r.fine_prob, (nf,), "<f4") if nf else torch.zeros(0, device="cuda")}
+        u16, i32, f32 = torch.uint16, torch.int32, torch.float32
+        return _copied({"codes_q": (r.codes_q, (n, 64), u16), "codes_r": (r.codes_r, (n, 64), u16),
+                        "lse_row": (r.lse_row, (n,), f32), "lse_col": (r.lse_col, (n,), f32),
+                        "row_best": (r.row_best, (n,), i32), "col_best": (r.col_best, (n,), i32),
+                        "coarse": (r.coarse, (nc, 2), i32), "coarse_prob": (r.coarse_prob, (nc,), f32),
+                        "fine": (r.fine, (nf, 3), i32), "fine_prob": (r.fine_prob, (nf,), f32)})
 
 
 # ---- dense PnP + RANSAC (Sec. 3.4, Eq. 10) ------------------------------------------------------
@@ -805,16 +815,14 @@ class PnP:
         r = self.solve_raw(cam, T_render, depth, alpha, matches, words, tau, min_alpha, refine_iters)
         K, nh = int(matches.shape[0]), int(words.shape[0])
         nv = r.n_valid
-        v = lambda p, shape, t: torch.as_tensor(_DevView(p, shape, t), device="cuda").clone()
-        empty = lambda shape, dt: torch.zeros(shape, dtype=dt, device="cuda")
-        return {"T": np.array(r.T_cw[:], np.float64).reshape(4, 4), "n_valid": nv, "n_inliers": r.n_inliers,
-                "best": (r.best_hypothesis, r.best_solution), "best_count": r.best_count,
-                "refine_steps": r.refine_steps,
-                "inlier": v(r.inlier, (K,), "|u1") if K else empty((0,), torch.uint8),
-                "valid_index": v(r.valid_index, (nv,), "<i4") if nv else empty((0,), torch.int32),
-                "points": v(r.points, (nv, 3), "<f8") if nv else empty((0, 3), torch.float64),
-                "hyp_counts": v(r.hyp_counts, (nh, 4), "<i4") if nh else empty((0, 4), torch.int32),
-                "hyp_poses": v(r.hyp_poses, (nh, 4, 12), "<f8") if nh else empty((0, 4, 12), torch.float64)}
+        out = {"T": np.array(r.T_cw[:], np.float64).reshape(4, 4), "n_valid": nv, "n_inliers": r.n_inliers,
+               "best": (r.best_hypothesis, r.best_solution), "best_count": r.best_count,
+               "refine_steps": r.refine_steps}
+        out.update(_copied({"inlier": (r.inlier, (K,), torch.uint8), "valid_index": (r.valid_index, (nv,), torch.int32),
+                            "points": (r.points, (nv, 3), torch.float64),
+                            "hyp_counts": (r.hyp_counts, (nh, 4), torch.int32),
+                            "hyp_poses": (r.hyp_poses, (nh, 4, 12), torch.float64)}))
+        return out
 
 
 # ---- dense stage with Algorithm 2's consistency check ------------------------------------------
