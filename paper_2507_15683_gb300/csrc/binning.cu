@@ -15,7 +15,7 @@ constexpr int kScanPer = 8;                             // counts per thread and
 constexpr int kScanChunk = kScanThreads * kScanPer;     // counts per chunk (32 KB of shared memory)
 static_assert(kScanPer == 8, "a thread reads and writes its counts as two 16-byte vectors");
 
-// Exclusive scan of tile_count[0..n) into tile_offset[0..n] and tile_cursor,
+// Exclusive scan of the n tile counters into tile_offset[0..n] and, in place, the counters,
 // by one CTA, in chunks of kScanChunk counts with a 64-bit carry: coalesced
 // loads into shared memory, each thread then sums kScanPer consecutive counts,
 // a block scan of those sums, and coalesced stores of the offsets. Also
@@ -32,12 +32,7 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_tiles(Work w) {
 #pragma unroll
     for (int i = 0; i < kScanPer; ++i) {
       const uint32_t k = base + (uint32_t)(i * kScanThreads + tid);
-      sv[i * kScanThreads + tid] = k < n ? w.tile_count[k] : 0u;
-    }
-#pragma unroll
-    for (int i = 0; i < kScanPer; ++i) {  // the next call counts from zero
-      const uint32_t k = base + (uint32_t)(i * kScanThreads + tid);
-      if (k < n) w.tile_count[k] = 0u;
+      sv[i * kScanThreads + tid] = k < n ? w.tile_ctr[(size_t)k << w.ctr_shift] : 0u;
     }
     __syncthreads();
     // this thread's kScanPer consecutive counts, as two 16-byte reads
@@ -92,7 +87,7 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_tiles(Work w) {
       if (k < n) {
         const uint32_t o = sv[i * kScanThreads + tid];
         w.tile_offset[k] = o;
-        w.tile_cursor[k] = o;
+        w.tile_ctr[(size_t)k << w.ctr_shift] = o;
       }
     }
     __syncthreads();  // sv and s_carry are reused by the next chunk
@@ -169,7 +164,7 @@ __global__ void __launch_bounds__(256) k_scatter(const View* __restrict__ views,
           const uint32_t wdt = x1 - x0 + 1u;
           const uint32_t ty = y0 + local / wdt, tx = x0 + local % wdt;
           const View& V = views[mm.z];
-          pos[u] = atomicAdd(&w.tile_cursor[V.tile_base + ty * (uint32_t)V.tiles_x + tx], 1u);
+          pos[u] = atomicAdd(&w.tile_ctr[(size_t)(V.tile_base + ty * (uint32_t)V.tiles_x + tx) << w.ctr_shift], 1u);
           val[u] = make_uint2(mm.w, base + (uint32_t)o);
         }
       }
@@ -323,6 +318,9 @@ __device__ void warp_sort_list(uint2* __restrict__ list, int n, const float4* __
 __global__ void __launch_bounds__(256, 4) k_sort_tiles(Work w) {
   __shared__ uint32_t s_rec[8][kWarpSortMax];
   pdl_wait();
+  // the next call counts from zero
+  for (uint32_t t = blockIdx.x * blockDim.x + threadIdx.x; t < w.n_tiles; t += gridDim.x * blockDim.x)
+    w.tile_ctr[(size_t)t << w.ctr_shift] = 0u;
   if (w.ctr->overflow) return;
   const int lane = threadIdx.x & 31;
   uint32_t* srec = s_rec[threadIdx.x >> 5];

@@ -170,12 +170,12 @@ struct gs_scene {
   // workspace
   DevBuf rec_a, rec_b, rec_c, rec_m, rec_j;
   uint32_t rec_cap = 0, jac_cap = 0;
-  DevBuf tile_count, tile_offset, tile_cursor, partials, chunks;
+  DevBuf tile_ctr, tile_offset, partials, chunks;
   uint32_t tile_cap = 0;
   DevBuf pairs, pairs_tmp;
   uint32_t pair_cap = 0;
   DevBuf result, views;     // views: the call table (counters, index ranges, views)
-  bool counts_zero = false;  // tile_count is all zeros (the scan leaves it so)
+  bool counts_zero = false;  // tile_ctr is all zeros (the sort leaves it so)
   Counters* ctr_host = nullptr;
   double* result_host = nullptr;
   // loss targets uploaded from host memory (gs_render_pose_grad_host) on a side
@@ -269,10 +269,10 @@ Work work_of(gs_scene* s, uint32_t n_tiles) {
   w.rec_j = dp<float>(s->rec_j);
   w.rec_cap = s->rec_cap;
   w.rec_seg = s->rec_cap / kRecRegions;
-  w.tile_count = dp<uint32_t>(s->tile_count);
+  w.tile_ctr = dp<uint32_t>(s->tile_ctr);
   w.tile_offset = dp<uint32_t>(s->tile_offset);
-  w.tile_cursor = dp<uint32_t>(s->tile_cursor);
   w.n_tiles = n_tiles;
+  w.ctr_shift = ctr_shift(n_tiles);
   w.pairs = dp<uint2>(s->pairs);
   w.pairs_tmp = dp<uint2>(s->pairs_tmp);
   w.pair_cap = s->pair_cap;
@@ -319,9 +319,8 @@ gs_status grow_tiles(gs_scene* s, uint64_t n_tiles) {
   if (n_tiles + 1 > s->tile_cap) {
     const uint64_t cap = n_tiles + 1;
     s->counts_zero = false;
-    GS_TRY(ensure(s->tile_count, cap * sizeof(uint32_t)));
+    GS_TRY(ensure(s->tile_ctr, ctr_words(cap) * sizeof(uint32_t)));
     GS_TRY(ensure(s->tile_offset, cap * sizeof(uint32_t)));
-    GS_TRY(ensure(s->tile_cursor, cap * sizeof(uint32_t)));
     GS_TRY(ensure(s->partials, cap * kPartialStride * sizeof(double)));
     GS_TRY(ensure(s->chunks, cap * (kPartialStride * sizeof(double) + sizeof(uint32_t))));
     s->tile_cap = (uint32_t)cap;
@@ -423,11 +422,11 @@ void fill_table(const gs_scene* s, const std::vector<View>& hv, const std::vecto
   std::memcpy(dst + table_views_off(s), hv.data(), hv.size() * sizeof(View));
 }
 
-// The per-tile counts start at zero: the scan leaves them so, and they are only
-// cleared here when they are new or a call failed between the two.
+// The tile counters start at zero: the sort leaves them so, and they are only
+// cleared here when they are new or a call failed on the way there.
 gs_status zero_counts(gs_scene* s, cudaStream_t st) {
   if (s->counts_zero) return GS_OK;
-  GS_CUDA(cudaMemsetAsync(s->tile_count.p, 0, (size_t)s->tile_cap * sizeof(uint32_t), st));
+  GS_CUDA(cudaMemsetAsync(s->tile_ctr.p, 0, ctr_words(s->tile_cap) * sizeof(uint32_t), st));
   s->counts_zero = true;
   return GS_OK;
 }
@@ -495,7 +494,7 @@ gs_status enqueue(gs_scene* s, const std::vector<View>& hv, const std::vector<in
   const int mode = g ? kModeTan : (feats && s->feat_dim) ? kModeFwdFeat : kModeFwd;
   const int grid = s->sm_count * std::max(1, cfg.grid_mult[mode]);  // projection, shading, scatter, sort
   GS_CUDA(mark(0));
-  if (!graph) s->counts_zero = false;  // until the scan is on the stream
+  if (!graph) s->counts_zero = false;  // until the sort is on the stream
   GS_CUDA(launch_project(sc, dviews, nv, w, grid, st));
   GS_CUDA(mark(1));
   // The shading pass reads only what the projection wrote, and the binning
@@ -522,11 +521,11 @@ gs_status enqueue(gs_scene* s, const std::vector<View>& hv, const std::vector<in
   // Jacobian the waiting blocks hold registers that the shading needs (gradient
   // 634 -> 648 us, visibility check 680 -> 703 us).
   GS_CUDA(launch_scan_tiles(w, st, !jac));
-  if (!graph) s->counts_zero = true;
   GS_CUDA(mark(3));
   GS_CUDA(launch_scatter(dviews, w, grid, st, !jac));
   GS_CUDA(mark(4));
   GS_CUDA(launch_sort_tiles(w, grid, st, !jac));
+  if (!graph) s->counts_zero = true;
   if (fork) GS_CUDA(cudaStreamWaitEvent(st, s->ev_shade, 0));
   GS_CUDA(mark(5));
   if (!g || feats) GS_CUDA(launch_composite(sc, dviews, nv, w, feats, cfg, s->sm_count, st));
@@ -1102,7 +1101,7 @@ void gs_destroy_scene(gs_scene* s) {
   for (auto& ev : s->ev_free)
     for (cudaEvent_t e : ev) cudaEventDestroy(e);
   for (DevBuf* b : {&s->pos, &s->cov, &s->sh, &s->feat, &s->rec_a, &s->rec_b, &s->rec_c, &s->rec_m, &s->rec_j,
-                    &s->tile_count, &s->tile_offset, &s->tile_cursor, &s->partials, &s->chunks, &s->pairs, &s->pairs_tmp,
+                    &s->tile_ctr, &s->tile_offset, &s->partials, &s->chunks, &s->pairs, &s->pairs_tmp,
                     &s->result, &s->views, &s->vis_T, &s->vis_last, &s->vis_acc, &s->vis_uv, &s->vis_blk})
     release(*b);
   for (void* h : {(void*)s->h_pos, (void*)s->h_cov, (void*)s->h_sh, (void*)s->h_feat})

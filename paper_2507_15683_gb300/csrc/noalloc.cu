@@ -52,9 +52,8 @@ struct Layout {
   static constexpr size_t rec_c = align256(rec_b + G * sizeof(float4));
   static constexpr size_t rec_m = align256(rec_c + G * sizeof(float4));
   static constexpr size_t tcount = align256(rec_m + G * sizeof(uint4));
-  static constexpr size_t toffset = align256(tcount + TL * sizeof(uint32_t));
-  static constexpr size_t tcursor = align256(toffset + TL * sizeof(uint32_t));
-  static constexpr size_t pairs = align256(tcursor + TL * sizeof(uint32_t));
+  static constexpr size_t toffset = align256(tcount + ctr_words(TL) * sizeof(uint32_t));
+  static constexpr size_t pairs = align256(toffset + TL * sizeof(uint32_t));
   static constexpr size_t pairs_tmp = align256(pairs + P * sizeof(uint2));
   static constexpr size_t ctr = align256(pairs_tmp + P * sizeof(uint2));
   static constexpr size_t view = align256(ctr + sizeof(Counters));
@@ -178,10 +177,10 @@ extern "C" gs_status gs_render_noalloc(const gs_scene_desc* d, const gs_camera* 
   // Gaussians whatever the SM count, so a segment takes the records of two
   // blocks, at most 2 x 256 = 512 = rec_cap / 64, and cannot overflow.
   w.rec_seg = GS_NOALLOC_MAX_GAUSSIANS / kRecRegions;
-  w.tile_count = reinterpret_cast<uint32_t*>(base + Layout::tcount);
+  w.tile_ctr = reinterpret_cast<uint32_t*>(base + Layout::tcount);
   w.tile_offset = reinterpret_cast<uint32_t*>(base + Layout::toffset);
-  w.tile_cursor = reinterpret_cast<uint32_t*>(base + Layout::tcursor);
   w.n_tiles = (uint32_t)n_tiles;
+  w.ctr_shift = ctr_shift((uint64_t)n_tiles);
   w.pairs = reinterpret_cast<uint2*>(base + Layout::pairs);
   w.pairs_tmp = reinterpret_cast<uint2*>(base + Layout::pairs_tmp);
   w.pair_cap = GS_NOALLOC_MAX_PAIRS;
@@ -201,7 +200,7 @@ extern "C" gs_status gs_render_noalloc(const gs_scene_desc* d, const gs_camera* 
   sc.feat_dim = d->feat_dim;
 
   // the scratch keeps the previous call's contents: reset what must start at zero
-  NA_CUDA(cudaMemsetAsync(w.tile_count, 0, (n_tiles + 1) * sizeof(uint32_t), st));
+  NA_CUDA(cudaMemsetAsync(w.tile_ctr, 0, ((size_t)n_tiles << w.ctr_shift) * sizeof(uint32_t), st));
   NA_CUDA(cudaMemsetAsync(w.ctr, 0, sizeof(Counters), st));
   NA_CUDA(cudaMemcpyAsync(dview, &V, sizeof(View), cudaMemcpyHostToDevice, st));
   NA_CUDA(cudaMemcpyAsync(dranges, hranges, sizeof(hranges), cudaMemcpyHostToDevice, st));
