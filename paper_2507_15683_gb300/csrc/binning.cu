@@ -130,7 +130,7 @@ __global__ void __launch_bounds__(256) k_scatter(const View* __restrict__ views,
     uint4 m = make_uint4(0u, 0u, 0u, 0u);
     if (r < w.rec_cap) {
       const uint32_t reg = r / w.rec_seg, loc = r - reg * w.rec_seg;
-      if (loc < min(w.ctr->rec_region[reg], w.rec_seg)) {
+      if (loc < min(w.ctr->rec_region[reg].n, w.rec_seg)) {
         m = w.rec_m[r];
         cnt = ((m.x >> 16) - (m.x & 0xffffu) + 1u) * ((m.y >> 16) - (m.y & 0xffffu) + 1u);
       }

@@ -697,7 +697,7 @@ gs_status prepare_call(gs_scene* s, const std::vector<View>& hv, cudaStream_t st
 // Record capacity the last call needed: every segment must hold its count.
 uint64_t records_capacity_needed(const Counters& c) {
   uint64_t mx = 0;
-  for (int k = 0; k < kRecRegions; ++k) mx = std::max<uint64_t>(mx, c.rec_region[k]);
+  for (int k = 0; k < kRecRegions; ++k) mx = std::max<uint64_t>(mx, c.rec_region[k].n);
   return mx * kRecRegions;
 }
 
@@ -706,7 +706,7 @@ std::vector<uint32_t> filled_records(const Counters& c, uint32_t rec_cap) {
   std::vector<uint32_t> idx;
   const uint32_t seg = rec_cap / kRecRegions;
   for (int k = 0; k < kRecRegions; ++k)
-    for (uint32_t j = 0; j < std::min(c.rec_region[k], seg); ++j) idx.push_back(k * seg + j);
+    for (uint32_t j = 0; j < std::min(c.rec_region[k].n, seg); ++j) idx.push_back(k * seg + j);
   return idx;
 }
 

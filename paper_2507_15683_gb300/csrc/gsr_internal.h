@@ -55,7 +55,9 @@ struct View {
 // serialises the whole grid. rec_region[k] may exceed the segment size (then
 // the overflow bit is set and the count tells the host how much to grow).
 struct Counters {
-  unsigned int rec_region[kRecRegions];  // records requested per segment
+  struct alignas(32) {     // one 32-byte sector each: the L2 takes atomics on a sector one after another
+    unsigned int n;        // records requested
+  } rec_region[kRecRegions];
   unsigned int pair_total;  // pairs requested by the binning
   unsigned int overflow;    // bit 0: records, bit 1: pairs, bit 2: pair count >= 2^32
   unsigned int fwd_queue;   // persistent tile queue of the forward render

@@ -382,7 +382,7 @@ __global__ void __launch_bounds__(kTileThreads, kProjResident)
     // warp-aggregated append into this block's record segment
     unsigned slot0 = 0;
     const int leader = __ffs(vmask) - 1;
-    if (lane == leader) slot0 = atomicAdd(&w.ctr->rec_region[region], (unsigned)__popc(vmask));
+    if (lane == leader) slot0 = atomicAdd(&w.ctr->rec_region[region].n, (unsigned)__popc(vmask));
     slot0 = __shfl_sync(0xffffffffu, slot0, leader);
     const unsigned local = slot0 + __popc(vmask & lt_mask);
     if (vis && local >= w.rec_seg) {
@@ -509,7 +509,7 @@ __global__ void __launch_bounds__(256, 3) k_shade(SceneDev sc, const View* __res
   if (w.ctr->overflow) return;
   for (uint32_t slot = blockIdx.x * blockDim.x + threadIdx.x; slot < w.rec_cap; slot += gridDim.x * blockDim.x) {
     const uint32_t reg = slot / w.rec_seg, loc = slot - reg * w.rec_seg;
-    if (loc >= min(w.ctr->rec_region[reg], w.rec_seg)) continue;
+    if (loc >= min(w.ctr->rec_region[reg].n, w.rec_seg)) continue;
     const float4 ra = w.rec_a[slot];
     const int i = __float_as_int(w.rec_b[slot].w);
     const uint4 m = w.rec_m[slot];
@@ -745,7 +745,7 @@ __global__ void __launch_bounds__(256) k_vis_chain(const View* __restrict__ view
     bool keep = false;
     if (slot < w.rec_cap) {
       const uint32_t reg = slot / w.rec_seg, loc = slot - reg * w.rec_seg;
-      if (loc < min(w.ctr->rec_region[reg], w.rec_seg)) {
+      if (loc < min(w.ctr->rec_region[reg].n, w.rec_seg)) {
         const float4 a0 = reinterpret_cast<const float4*>(acc)[2 * (size_t)slot];
         const float4 a1 = reinterpret_cast<const float4*>(acc)[2 * (size_t)slot + 1];
         if (a0.x != 0.0f || a0.y != 0.0f || a0.z != 0.0f || a0.w != 0.0f || a1.x != 0.0f || a1.y != 0.0f) {
