@@ -12,7 +12,7 @@ namespace gsr {
 constexpr int kTile = 16;          // tile edge in pixels
 constexpr int kTileThreads = 256;  // one thread per pixel of a tile
 constexpr int kSortCap = 2048;     // (tile, Gaussian) pairs a tile sorts in shared memory
-constexpr int kJacStride = 48;     // floats per record of the pose Jacobian (45 used)
+constexpr int kJacStride = 44;     // floats per record of the pose Jacobian and colour
 constexpr int kPartialStride = 8;  // doubles per tile partial (loss + 6 grad + pad)
 constexpr int kChunkTiles = 64;    // tiles per first-level chunk of the fp64 pose reduction
 constexpr int kWarpSortMax = 256;  // longest tile list sorted by one warp (registers)

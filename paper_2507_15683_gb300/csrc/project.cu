@@ -500,6 +500,9 @@ __global__ void __launch_bounds__(kTileThreads, kProjResident)
   }
 }
 
+// Place of d colour_ch / d rho_d in a Jacobian record.
+__host__ __device__ constexpr int jac_colour(int ch, int d) { return d == 2 ? 38 + ch : (ch == 0 ? 10 : ch == 1 ? 34 : 36) + d; }
+
 // ---------------------------------------------------------------------------
 // Shading pass over the compact records: conic, SH colour, float-float
 // blending centre and, for the pose gradient, the per-record pose Jacobian.
@@ -664,11 +667,15 @@ __global__ void __launch_bounds__(256, 3) k_shade(SceneDev sc, const View* __res
       // (0,1), (2,3), (4,5). With the pixel offset (dx, dy) = centre - pixel,
       //   -dpower/dxi = dx (A du + B dv) + dy (B du + C dv) + dx^2 dA/2
       //                 + dx dy dB + dy^2 dC/2,
-      // so pair k holds three float4: (P, Q), (dA/2, dB), (dC/2, dz), each
-      // as the two directions of the pair, with P = A du + B dv and
-      // Q = B du + C dv; then d(r, g, b)/d rho in three float4 (three
-      // directions and a zero).
-      float jt[48];
+      // so pair k holds (P, Q), (dA/2, dB) and dC/2, each as the two
+      // directions of the pair, with P = A du + B dv and Q = B du + C dv, in
+      // two and a half float4. The other halves hold d(r, g)/d rho_0..1 and
+      // the two entries of dz that are not 0 or 1 (dz/dphi_0 = py,
+      // dz/dphi_1 = -px), and two more float4 the rest of the colour rows and
+      // the colour: 11 float4, every word used. With dz in full, zeros behind
+      // the colour rows and the colour apart they were 13, and a blended hit
+      // reads each of them into every lane: JAC_NEW.
+      float jt[kJacStride];
 #pragma unroll
       for (int k = 0; k < 3; ++k) {
 #pragma unroll
@@ -679,18 +686,19 @@ __global__ void __launch_bounds__(256, 3) k_shade(SceneDev sc, const View* __res
           jt[12 * k + 4 + h] = 0.5f * jac[12 + d];
           jt[12 * k + 6 + h] = jac[18 + d];
           jt[12 * k + 8 + h] = 0.5f * jac[24 + d];
-          jt[12 * k + 10 + h] = jac[30 + d];
         }
       }
+      jt[22] = jac[33];  // dz/dphi_0, dz/dphi_1
+      jt[23] = jac[34];
 #pragma unroll
       for (int ch = 0; ch < 3; ++ch) {
 #pragma unroll
-        for (int k = 0; k < 3; ++k) jt[36 + 4 * ch + k] = jac[36 + 3 * ch + k];
-        jt[39 + 4 * ch] = 0.0f;
+        for (int k = 0; k < 3; ++k) jt[jac_colour(ch, k)] = jac[36 + 3 * ch + k];
+        jt[41 + ch] = rgb[ch];
       }
       float4* jo = reinterpret_cast<float4*>(w.rec_j + (size_t)slot * kJacStride);
 #pragma unroll
-      for (int q = 0; q < 12; ++q) jo[q] = make_float4(jt[4 * q], jt[4 * q + 1], jt[4 * q + 2], jt[4 * q + 3]);
+      for (int q = 0; q < kJacStride / 4; ++q) jo[q] = make_float4(jt[4 * q], jt[4 * q + 1], jt[4 * q + 2], jt[4 * q + 3]);
     }
   }
 }
@@ -755,7 +763,7 @@ __global__ void __launch_bounds__(256) k_vis_chain(const View* __restrict__ view
           for (int d = 0; d < 3; ++d) {
             const int o = 12 * (d >> 1) + (d & 1);  // direction d of pair d / 2
             const float sp = J[o] * a0.x + J[o + 2] * a0.y + J[o + 4] * a0.z + J[o + 6] * a0.w + J[o + 8] * a1.x;
-            gr[d] = (J[36 + d] + J[40 + d] + J[44 + d]) * a1.y - sp;
+            gr[d] = (J[jac_colour(0, d)] + J[jac_colour(1, d)] + J[jac_colour(2, d)]) * a1.y - sp;
           }
           float g[3];
 #pragma unroll

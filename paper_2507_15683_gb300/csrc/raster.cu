@@ -458,7 +458,7 @@ __global__ void __launch_bounds__(kTileThreads, MINB) k_composite(SceneDev sc, c
   if (FEAT) {  // empty slots multiply stale rows by zero weights: keep the rows finite
     for (int i = threadIdx.x & 31; i < kSlots * kFbRow; i += 32) fb[i] = 0;
   }
-  float4* sj = reinterpret_cast<float4*>(smem_raw + kSmJac);  // TAN: KB x 12
+  float4* sj = reinterpret_cast<float4*>(smem_raw + kSmJac);  // TAN: KB x 11
   __shared__ uint32_t s_tile;
   __shared__ uint32_t s_tmp[kWarps];
   __shared__ float s_red[kWarps][8];
@@ -585,7 +585,7 @@ __global__ void __launch_bounds__(kTileThreads, MINB) k_composite(SceneDev sc, c
       if (__syncthreads_count(done) == kTileThreads) break;
       const int bn = min(kB, n - bs);
       if (TAN) {
-        // Pose Jacobians (bn x 12 float4) by cp.async, without registers:
+        // Pose Jacobians (bn x 11 float4) by cp.async, without registers:
         // consecutive threads copy consecutive 16-byte pieces of a record; the
         // list entries of all of a thread's pieces are loaded first.
         constexpr int kJ4 = kJacStride / 4;
@@ -614,7 +614,6 @@ __global__ void __launch_bounds__(kTileThreads, MINB) k_composite(SceneDev sc, c
           if (part == 0) {
             sa[e] = a;
             sb[e] = bb;
-            scol[e] = cc;
           }
           smask[part * kB + e] = warp_hit_mask(a, bb.x, floor_threshold(bb.y), part * kPW, part * kPW + kPW);
         }
@@ -645,13 +644,19 @@ __global__ void __launch_bounds__(kTileThreads, MINB) k_composite(SceneDev sc, c
         const bool stop = take && (Tn < kTCut);
         const bool acc = take && !stop;
         const float wgt = acc ? __fmul_rn(alpha, T) : 0.0f;
-        const float4 c = scol[j];
-        if (TAN) {
-          // staged Jacobian: per direction pair k, (P, Q), (dA/2, dB),
-          // (dC/2, dz) with P = A du + B dv, Q = B du + C dv; then the colour
-          // rows. S_k = dx P + dy Q + dx^2 dA/2 + dx dy dB + dy^2 dC/2 is
+        float3 c;
+        if (!TAN) {
+          const float4 cc = scol[j];
+          c = make_float3(cc.x, cc.y, cc.z);
+        } else {
+          // staged Jacobian: per direction pair k, (P, Q), (dA/2, dB), dC/2
+          // with P = A du + B dv, Q = B du + C dv and half a float4 of other
+          // entries; then the rest of the colour rows, and the colour.
+          // S_k = dx P + dy Q + dx^2 dA/2 + dx dy dB + dy^2 dC/2 is
           // -dpower/dxi_k.
           const float4* J4 = sj + j * (kJacStride / 4);
+          const float4 e10 = J4[10];
+          c = make_float3(e10.y, e10.z, e10.w);
           // T dalpha = -alpha T S (0 where the 0.99 cap is active); -alpha T
           // is folded into the monomials of the pixel offset
           const float nat = (acc && oe < kAlphaCap) ? -alpha * T : 0.0f;
@@ -663,6 +668,7 @@ __global__ void __launch_bounds__(kTileThreads, MINB) k_composite(SceneDev sc, c
           const float2 AE = make_float2(ae, ae);
           const float2 CR = make_float2(c.x, c.x), CG = make_float2(c.y, c.y), CB = make_float2(c.z, c.z);
           const float2 ZZ = make_float2(zj, zj), WW = make_float2(wgt, wgt);
+          float dzp1 = 0.0f;  // dz/dphi_1
 #pragma unroll
           for (int k = 0; k < 3; ++k) {
             const float4 pq = J4[3 * k], ab = J4[3 * k + 1], cz = J4[3 * k + 2];
@@ -676,17 +682,23 @@ __global__ void __launch_bounds__(kTileThreads, MINB) k_composite(SceneDev sc, c
             dC0[k] = __ffma2_rn(dw, CR, dC0[k]);
             dC1[k] = __ffma2_rn(dw, CG, dC1[k]);
             dC2[k] = __ffma2_rn(dw, CB, dC2[k]);
-            // dz/drho_0 = dz/drho_1 = 0: the first pair has no w dz term
-            dD[k] = __ffma2_rn(dw, ZZ, k == 0 ? dD[k] : __ffma2_rn(make_float2(cz.z, cz.w), WW, dD[k]));
+            // dz/drho = (0, 0, 1), dz/dphi = (py, -px, 0)
+            if (k == 1) {
+              dD[1].x = __fadd_rn(wgt, dD[1].x);
+              dD[1].y = fmaf(cz.z, wgt, dD[1].y);
+              dzp1 = cz.w;
+            }
+            if (k == 2) dD[2].x = fmaf(dzp1, wgt, dD[2].x);
+            dD[k] = __ffma2_rn(dw, ZZ, dD[k]);
+            // colour depends on the camera centre only: rho directions 0..2
+            if (k == 0) dC0[0] = __ffma2_rn(make_float2(cz.z, cz.w), WW, dC0[0]);
+            if (k == 2) dC1[0] = __ffma2_rn(make_float2(cz.z, cz.w), WW, dC1[0]);
           }
-          // colour depends on the camera centre only: rho directions 0..2
-          const float4 r0 = J4[9], r1 = J4[10], r2 = J4[11];
-          dC0[0] = __ffma2_rn(make_float2(r0.x, r0.y), WW, dC0[0]);
-          dC0[1].x = fmaf(r0.z, wgt, dC0[1].x);
-          dC1[0] = __ffma2_rn(make_float2(r1.x, r1.y), WW, dC1[0]);
-          dC1[1].x = fmaf(r1.z, wgt, dC1[1].x);
-          dC2[0] = __ffma2_rn(make_float2(r2.x, r2.y), WW, dC2[0]);
-          dC2[1].x = fmaf(r2.z, wgt, dC2[1].x);
+          const float4 e9 = J4[9];
+          dC2[0] = __ffma2_rn(make_float2(e9.x, e9.y), WW, dC2[0]);
+          dC0[1].x = fmaf(e9.z, wgt, dC0[1].x);
+          dC1[1].x = fmaf(e9.w, wgt, dC1[1].x);
+          dC2[1].x = fmaf(e10.x, wgt, dC2[1].x);
         }
         C0 = fmaf(wgt, c.x, C0);
         C1 = fmaf(wgt, c.y, C1);
