@@ -6,6 +6,7 @@
 #include <stdint.h>
 
 #include "gsr.h"
+#include "gsr_launch.h"
 
 namespace gsr {
 
@@ -153,29 +154,6 @@ struct LaunchCfg {
   int per_sm[kModeCount] = {0, 0, 0};
   int grid_mult[kModeCount] = {8, 8, 8};
 };
-
-// A kernel launched by launch_dependent may start (its blocks become resident)
-// before the kernel in front of it on the stream has ended, once all blocks of
-// that one have called pdl_trigger or exited; it calls pdl_wait before anything
-// else, which returns when that kernel has completed. So the launch and the
-// block scheduling of one kernel of a chain hide behind the last blocks of the
-// kernel before. Without `early` it is an ordinary launch. Every kernel launched this way waits on every path, so the
-// completion of one implies that of all kernels before it.
-__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-template <typename... P, typename... A>
-cudaError_t launch_dependent(bool early, void (*kernel)(P...), int grid, int block, cudaStream_t st, A... args) {
-  cudaLaunchAttribute attr;
-  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr.val.programmaticStreamSerializationAllowed = early ? 1 : 0;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)grid);
-  cfg.blockDim = dim3((unsigned)block);
-  cfg.stream = st;
-  cfg.attrs = &attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
-}
 
 // launchers (return the CUDA error of the launch)
 cudaError_t launch_pack_scene(const float* means, const float* scales, const float* quats,

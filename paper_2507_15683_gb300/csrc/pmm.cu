@@ -34,6 +34,7 @@
 #include <string>
 #include <type_traits>
 
+#include "gsr_launch.h"
 #include "gsr_pmm.h"
 
 namespace gsr {
@@ -370,6 +371,8 @@ __global__ void __launch_bounds__(kSumThreads, 2) k_pmm_sums(const unsigned char
                                                              int per, float s_exp, float* __restrict__ prow_v,
                                                              float* __restrict__ pcol_v, int* __restrict__ err,
                                                              int wait_limit) {
+  gsr::pdl_wait();
+  gsr::pdl_trigger();
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   SumSmem& S = *reinterpret_cast<SumSmem*>(smem_raw);
   const int t0 = (int)blockIdx.x * per, nt = min(per, (nb + 1) / 2 * nb - t0);
@@ -626,6 +629,8 @@ __global__ void __launch_bounds__(kRoleThreads, 2) k_pmm_argmax(const unsigned c
                                                                 const float* __restrict__ nlse_c,
                                                                 float* __restrict__ prow_v, int* __restrict__ prow_i,
                                                                 int* __restrict__ err, int wait_limit) {
+  gsr::pdl_wait();
+  gsr::pdl_trigger();
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   BestSmem& S = *reinterpret_cast<BestSmem*>(smem_raw);
   const int t0 = (int)blockIdx.x * per, nt = min(per, nb * nb - t0);
@@ -826,6 +831,8 @@ constexpr int kRedWarps = 8;
 __global__ void __launch_bounds__(kRedRows * kRedWarps) k_pmm_lse(const float* __restrict__ part, int nb, int n,
                                                                   float inv_tau, float* __restrict__ lse,
                                                                   float* __restrict__ nlse) {
+  gsr::pdl_wait();
+  gsr::pdl_trigger();
   __shared__ float sp[kRedWarps][kRedRows];
   const int lane = threadIdx.x & 31, g = threadIdx.x >> 5;
   const int i = blockIdx.x * kRedRows + lane;
@@ -849,6 +856,8 @@ __global__ void __launch_bounds__(kRedRows * kRedWarps) k_pmm_lse(const float* _
 // the best of a row's partials: two from each CTA that holds tiles of its row block
 __global__ void k_pmm_best(const float* __restrict__ pv, const int* __restrict__ pi, int nb, int per, int n,
                            int* __restrict__ best) {
+  gsr::pdl_wait();
+  gsr::pdl_trigger();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   const int rb = i / kTile, parts = 2 * ((rb * nb + nb - 1) / per - best_first(rb, nb, per) + 1);
@@ -898,6 +907,8 @@ __global__ void k_pmm_mnn(int n, const int* __restrict__ row_best, const int* __
                           const __nv_bfloat16* __restrict__ cq, const __nv_bfloat16* __restrict__ cr,
                           const float* __restrict__ lse_row, const float* __restrict__ lse_col, float s_two,
                           int* __restrict__ flag, float* __restrict__ prob, const int* __restrict__ err) {
+  gsr::pdl_wait();
+  gsr::pdl_trigger();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   if (*err) {
@@ -914,6 +925,8 @@ __global__ void k_pmm_mnn(int n, const int* __restrict__ row_best, const int* __
 __global__ void k_pmm_mnn_scatter(int n, const int* __restrict__ row_best, const int* __restrict__ flag,
                                   const int* __restrict__ off, const float* __restrict__ prob_in,
                                   int* __restrict__ coarse, float* __restrict__ prob) {
+  gsr::pdl_wait();
+  gsr::pdl_trigger();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n || !flag[i]) return;
   const int pos = off[i];
@@ -966,6 +979,8 @@ __global__ void __launch_bounds__(kWin, 8) k_pmm_fine(const __grid_constant__ CU
                                                       float s_two, int* __restrict__ slot_r, float* __restrict__ slot_p,
                                                       int* __restrict__ win_count, const int* __restrict__ n_coarse,
                                                       int* __restrict__ err) {
+  gsr::pdl_wait();
+  gsr::pdl_trigger();
   // the unit vectors, channel-major (query, then rendered); then the window's
   // exponentials; then its similarities
   __shared__ __align__(128) float buf[kWin * kEs];
@@ -1148,6 +1163,8 @@ constexpr int kScanSteps = 8;
 __global__ void __launch_bounds__(kScanThreads) k_pmm_scan(int n_win, const int* __restrict__ cnt,
                                                            int* __restrict__ off, int* __restrict__ total,
                                                            const int* __restrict__ n_dev) {
+  gsr::pdl_wait();
+  gsr::pdl_trigger();
   __shared__ uint32_t wsum[2][32];
   if (n_dev) n_win = *n_dev;  // a count produced on the device (the coarse matches)
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -1214,6 +1231,8 @@ constexpr int kScatterWins = 4;
 __global__ void __launch_bounds__(kScatterWins* kWin) k_pmm_fine_scatter(
     int W, int Wc, const int* __restrict__ coarse, const int* __restrict__ slot_r, const float* __restrict__ slot_p,
     const int* __restrict__ off, int* __restrict__ fine, float* __restrict__ prob, const int* __restrict__ n_coarse) {
+  gsr::pdl_wait();
+  gsr::pdl_trigger();
   __shared__ int first[kScatterWins];  // matches of each window's first warp
   const int wi = threadIdx.x / kWin, a = threadIdx.x % kWin, k = blockIdx.x * kScatterWins + wi;
   const bool in = k < *n_coarse;
@@ -1439,35 +1458,38 @@ gs_status gs_pmm_match(gs_pmm* m, const float* feat_query, const float* feat_ren
   // pass 1: row and column exp sums, then the log-sum-exps
   const int stiles = (nb + 1) / 2 * nb;
   const int sctas = std::min(stiles, 2 * m->sm_count), sper = (stiles + sctas - 1) / sctas;
-  k_pmm_sums<<<(stiles + sper - 1) / sper, kSumThreads, kSumSmemBytes, st>>>(m->paired_q, cr, n, nb, sper, s_exp,
-                                                                             m->prow_v, m->pcol_v, err, m->wait_limit);
-  PMM_CUDA(cudaGetLastError());
+  // every kernel from here on starts early: thirteen short and long ones in a
+  // row, whose launches and block scheduling hide behind one another (1080p maps
+  // 1331 -> 1301 us, three localisations of 960 x 540 views, with the solver's
+  // early starts, 2335 -> 2174 us)
+  auto go = [&](auto kernel, int grid, int block, size_t smem, auto... args) -> cudaError_t {
+    return gsr::launch_dependent(true, kernel, dim3((unsigned)grid), block, smem, st, args...);
+  };
+  PMM_CUDA(go(k_pmm_sums, (stiles + sper - 1) / sper, kSumThreads, kSumSmemBytes, m->paired_q, cr, n, nb, sper, s_exp,
+              m->prow_v, m->pcol_v, err, m->wait_limit));
   const int rd = nb * (kTile / kRedRows);
-  k_pmm_lse<<<rd, kRedRows * kRedWarps, 0, st>>>(m->prow_v, nb, n, inv_tau, m->lse_row, m->nlse_row);
-  k_pmm_lse<<<rd, kRedRows * kRedWarps, 0, st>>>(m->pcol_v, nb, n, inv_tau, m->lse_col, m->nlse_col);
+  PMM_CUDA(go(k_pmm_lse, rd, kRedRows * kRedWarps, 0, m->prow_v, nb, n, inv_tau, m->lse_row, m->nlse_row));
+  PMM_CUDA(go(k_pmm_lse, rd, kRedRows * kRedWarps, 0, m->pcol_v, nb, n, inv_tau, m->lse_col, m->nlse_col));
   // pass 2: row argmax of log P_M, then (operands swapped) its column argmax
   const int per = m->per, bgrid = (tiles + per - 1) / per;
-  k_pmm_argmax<<<bgrid, kRoleThreads, kBestSmemBytes, st>>>(cq, cr, n, nb, per, s_two, m->nlse_col, m->prow_v,
-                                                            m->prow_i, err, m->wait_limit);
-  k_pmm_best<<<rg, 256, 0, st>>>(m->prow_v, m->prow_i, nb, per, n, m->row_best);
-  k_pmm_argmax<<<bgrid, kRoleThreads, kBestSmemBytes, st>>>(cr, cq, n, nb, per, s_two, m->nlse_row, m->prow_v,
-                                                            m->prow_i, err, m->wait_limit);
-  k_pmm_best<<<rg, 256, 0, st>>>(m->prow_v, m->prow_i, nb, per, n, m->col_best);
-  PMM_CUDA(cudaGetLastError());
+  PMM_CUDA(go(k_pmm_argmax, bgrid, kRoleThreads, kBestSmemBytes, cq, cr, n, nb, per, s_two, m->nlse_col, m->prow_v,
+              m->prow_i, err, m->wait_limit));
+  PMM_CUDA(go(k_pmm_best, rg, 256, 0, m->prow_v, m->prow_i, nb, per, n, m->row_best));
+  PMM_CUDA(go(k_pmm_argmax, bgrid, kRoleThreads, kBestSmemBytes, cr, cq, n, nb, per, s_two, m->nlse_row, m->prow_v,
+              m->prow_i, err, m->wait_limit));
+  PMM_CUDA(go(k_pmm_best, rg, 256, 0, m->prow_v, m->prow_i, nb, per, n, m->col_best));
   // mutual nearest neighbours in ascending query order
-  k_pmm_mnn<<<rg, 256, 0, st>>>(n, m->row_best, m->col_best, m->codes_q, m->codes_r, m->lse_row, m->lse_col, s_two,
-                                m->win_cnt, m->slot_p, err);
-  k_pmm_scan<<<1, kScanThreads, 0, st>>>(n, m->win_cnt, m->win_off, m->counters, nullptr);
-  k_pmm_mnn_scatter<<<rg, 256, 0, st>>>(n, m->row_best, m->win_cnt, m->win_off, m->slot_p, m->coarse, m->coarse_p);
-  PMM_CUDA(cudaGetLastError());
+  PMM_CUDA(go(k_pmm_mnn, rg, 256, 0, n, m->row_best, m->col_best, m->codes_q, m->codes_r, m->lse_row, m->lse_col,
+              s_two, m->win_cnt, m->slot_p, err));
+  PMM_CUDA(go(k_pmm_scan, 1, kScanThreads, 0, n, m->win_cnt, m->win_off, m->counters, nullptr));
+  PMM_CUDA(go(k_pmm_mnn_scatter, rg, 256, 0, n, m->row_best, m->win_cnt, m->win_off, m->slot_p, m->coarse, m->coarse_p));
   // fine level without a round trip: one CTA per cell (the most coarse matches
   // there can be); those past the device-side coarse count return at once
-  k_pmm_fine<<<n, kWin, 0, st>>>(map_q, map_r, m->W, m->Wc, m->coarse, inv_tau, s_exp, s_two, m->slot_r, m->slot_p,
-                                 m->win_cnt, m->counters, err);
-  k_pmm_scan<<<1, kScanThreads, 0, st>>>(0, m->win_cnt, m->win_off, m->counters + 1, m->counters);
-  k_pmm_fine_scatter<<<(n + kScatterWins - 1) / kScatterWins, kScatterWins * kWin, 0, st>>>(
-      m->W, m->Wc, m->coarse, m->slot_r, m->slot_p, m->win_off, m->fine, m->fine_p, m->counters);
-  PMM_CUDA(cudaGetLastError());
+  PMM_CUDA(go(k_pmm_fine, n, kWin, 0, map_q, map_r, m->W, m->Wc, m->coarse, inv_tau, s_exp, s_two, m->slot_r,
+              m->slot_p, m->win_cnt, m->counters, err));
+  PMM_CUDA(go(k_pmm_scan, 1, kScanThreads, 0, 0, m->win_cnt, m->win_off, m->counters + 1, m->counters));
+  PMM_CUDA(go(k_pmm_fine_scatter, (n + kScatterWins - 1) / kScatterWins, kScatterWins * kWin, 0, m->W, m->Wc, m->coarse,
+              m->slot_r, m->slot_p, m->win_off, m->fine, m->fine_p, m->counters));
   PMM_CUDA(cudaMemcpyAsync(m->host, m->counters, 4 * sizeof(int), cudaMemcpyDeviceToHost, st));
   PMM_CUDA(cudaStreamSynchronize(st));
   if (m->host[3])
