@@ -764,7 +764,7 @@ def bench_pmm(gsr, synth, torch, pk_src, steps, warmup, with_oracle=False):
     sims = float(n) * n
     mma_flops = 3 * 2 * 2 * 32 * sims  # three split products, two passes over the tiles, K = 32
     sm = torch.cuda.get_device_properties(0).multi_processor_count
-    mufu_peak = sm * 16 * float(pk.get("sm_max_mhz", 2070.0)) * 1e6  # exp2 per second (16 per SM per clock)
+    mufu_peak = sm * 32 * float(pk.get("sm_max_mhz", 2070.0)) * 1e6  # exp2 per second (32 per SM per clock, measured)
     decisions = pmm_decisions(gsr, synth, torch, scene, T_ref, T_q) if with_oracle else None
     return {"workload": "PMM of 1920x1080 32-channel feature maps rendered from 1M Gaussians (query 2 deg / 5 m "
                         "off the reference): 8x8 coarse cells, tau 0.1, coarse MNN + 8x8-window fine MNN",

@@ -101,7 +101,7 @@ typedef struct {
 } gs_outputs;
 
 /* Batch flags */
-#define GS_BATCH_GRAPH 1u      /* capture the batch once into a CUDA graph and replay it */
+#define GS_BATCH_GRAPH 1u      /* replay the batch from a CUDA graph, captured once per set of view sizes */
 
 /* Create a scene (Sec. 3.1). Packs the Gaussians into the device layout used by
  * the kernels (centre + max scale, binary32 3D covariance + opacity, SH
@@ -178,9 +178,11 @@ gs_status gs_render_pose_grad_async(gs_scene* scene, const gs_camera* cam, const
  * n_views entries (outs hold device pointers). Each view's outputs equal those
  * of gs_render for that view. flags: 0 = synchronous (regrow rule of
  * gs_render); GS_BATCH_GRAPH = asynchronous replay of a CUDA graph captured on
- * the first call for this (n_views, cams, outs) layout -- poses may change
- * between calls; reserve the workspace first (gs_scene_reserve) and check
- * gs_scene_status(). Errors: INVALID_ARG, OOM, CUDA. */
+ * the first call with these view sizes (and with or without feature maps) --
+ * poses, intrinsics and output pointers travel in the table that each replay
+ * uploads and may change between calls; reserve the workspace first
+ * (gs_scene_reserve) and check gs_scene_status(). Errors: INVALID_ARG, OOM,
+ * CUDA. */
 gs_status gs_render_batch(gs_scene* scene, int n_views, const gs_camera* cams, const gs_pose* poses,
                           const gs_outputs* outs, unsigned flags, void* stream);
 
@@ -195,10 +197,11 @@ gs_status gs_render_batch(gs_scene* scene, int n_views, const gs_camera* cams, c
  * flags 0: synchronous (regrow rule of gs_render); loss_out (host, n_views)
  * and grad_out (host, n_views x 6) are written when not NULL; results_dev,
  * when not NULL, also receives them. GS_BATCH_GRAPH: asynchronous replay of a
- * CUDA graph captured on the first call for this layout (cameras, outputs,
- * targets, weights, results_dev); poses may change between calls; results_dev
- * (device, n_views x 8 doubles: loss, 6 gradient entries, 0) is required and
- * loss_out / grad_out are not written. Errors: INVALID_ARG, OOM, CUDA. */
+ * CUDA graph captured on the first call with these view sizes and this
+ * results_dev; poses, intrinsics, outputs, targets and weights may change
+ * between calls; results_dev (device, n_views x 8 doubles: loss, 6 gradient
+ * entries, 0) is required and loss_out / grad_out are not written. Errors:
+ * INVALID_ARG, OOM, CUDA. */
 gs_status gs_render_pose_grad_batch(gs_scene* scene, int n_views, const gs_camera* cams, const gs_pose* poses,
                                     const float* const* target_rgb, const float* const* target_depth,
                                     const float* const* pixel_weight, float depth_weight, const gs_outputs* outs,
@@ -351,7 +354,7 @@ gs_status gs_scene_work_counts(gs_scene* scene, void* stream, int64_t* blended, 
  * No configuration changes a result: the blending order and every reduction
  * order are fixed by the tile lists, so every configuration gives the same
  * bits. Shapes without a configuration use the defaults. Changing one makes
- * the next graph-mode batch call capture its graph again. */
+ * the next replayed call capture its graph again. */
 #define GS_MODE_FORWARD 0     /* forward render without features */
 #define GS_MODE_FEATURES 1    /* forward render with the feature map */
 #define GS_MODE_POSE_GRAD 2   /* pose-gradient call (the tangent pass) */

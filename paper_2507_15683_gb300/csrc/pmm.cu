@@ -949,8 +949,8 @@ __global__ void k_pmm_mnn_scatter(int n, const int* __restrict__ row_best, const
 // wavefronts whatever its lanes share, so 64 accumulators from 16-byte
 // broadcasts of one side (306 us for 23,448 windows) lost to the 8 x 8 tile
 // (295 us), and loading the windows through registers cost more wavefronts than
-// the product. Now
-// 263 us; 418 us with the windows loaded through registers, a row pair per
+// the product. Now 263 us;
+// 418 us with the windows loaded through registers, a row pair per
 // thread against broadcast columns and the exponentials taken twice.
 // ---------------------------------------------------------------------------
 constexpr int kEs = kWin + 4;  // row stride of the 64 x 64 buffer: 16-byte rows, float4 reads by row conflict-free

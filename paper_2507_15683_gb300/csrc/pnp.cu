@@ -3,9 +3,9 @@
 //   1. lifting: every match whose rendered pixel has alpha >= min_alpha gets
 //      the world point R_r^T (z K^-1 (x + .5, y + .5, 1) - t_r), z = depth /
 //      alpha (fp64), compacted in match order;
-//   2. hypotheses: one thread per RANSAC sample solves P3P in fp64 (Grunert's
-//      quartic in v = s3 / s1, Ferrari's closed form polished by Newton,
-//      triad absolute orientation);
+//   2. hypotheses, beside the lifting: four lanes per RANSAC sample solve P3P
+//      in fp64 (Grunert's quartic in v = s3 / s1, Ferrari's closed form
+//      polished by Newton, triad absolute orientation), one solution each;
 //   3. scoring: every solution against every lifted match, packed fp32
 //      (__ffma2_rn on pairs of matches), inlier counts per solution;
 //   4. the RANSAC argmax (most inliers, lowest index on ties);
