@@ -1692,6 +1692,11 @@ gs_status gs_autotune(gs_scene* s, int mode, int n_views, const gs_camera* cams,
   return GS_OK;
 }
 
+// Number of a compositor variant in a saved file: files keep the numbers from
+// when the variants now numbered 0 and 2 of the forward and gradient modes
+// stood the other way round, so that a saved choice means the same kernel.
+static int file_variant(int mode, int v) { return mode != kModeFwdFeat && (v == 0 || v == 2) ? 2 - v : v; }
+
 gs_status gs_tune_save(const gs_scene* s, const char* path) {
   g_err.clear();
   GS_TRY(check_scene(s));
@@ -1719,7 +1724,7 @@ gs_status gs_tune_save(const gs_scene* s, const char* path) {
   for (const auto& e : s->launch)
     for (int m = 0; m < kModeCount; ++m)
       std::fprintf(f, "%s/%d|%d|%s|%d %d %d\n", s->device_name.c_str(), s->sm_count, m, e.first.c_str(),
-                   e.second.variant[m], e.second.per_sm[m], e.second.grid_mult[m]);
+                   file_variant(m, e.second.variant[m]), e.second.per_sm[m], e.second.grid_mult[m]);
   const bool ok = std::fclose(f) == 0;
   return ok ? GS_OK : fail(GS_ERR_INVALID_ARG, std::string("cannot write ") + path);
 }
@@ -1746,7 +1751,7 @@ gs_status gs_tune_load(gs_scene* s, const char* path, int* loaded) {
       st = fail(GS_ERR_INVALID_ARG, "malformed line in " + std::string(path) + ": " + l);
       break;
     }
-    st = set_cfg(s, mode, l.substr(b + 1, c - b - 1), v, p, gm);
+    st = set_cfg(s, mode, l.substr(b + 1, c - b - 1), file_variant(mode, v), p, gm);
     n += st == GS_OK;
   }
   std::fclose(f);
