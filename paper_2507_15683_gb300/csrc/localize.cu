@@ -49,7 +49,18 @@ gs_status gs_pose_difference(const gs_pose* T1, const gs_pose* T2, double* angle
   for (int i = 0; i < 3; ++i)
     for (int j = 0; j < 3; ++j) tr += A[4 * i + j] * B[4 * i + j];
   tr = std::min(3.0, std::max(tr, -1.0));
-  *angle_deg = std::acos((tr - 1.0) / 2.0) * (180.0 / M_PI);
+  const double c = (tr - 1.0) / 2.0;
+  double angle = std::acos(c);
+  if (c < -0.9999) {
+    // near a half turn the cosine alone leaves 1e-8 rad (rounding of the trace,
+    // which differs from one host to the next); the sine comes from the skew part
+    auto D = [&](int i, int j) {  // (R1 R2^T)_ij
+      return A[4 * i] * B[4 * j] + A[4 * i + 1] * B[4 * j + 1] + A[4 * i + 2] * B[4 * j + 2];
+    };
+    const double x = D(2, 1) - D(1, 2), y = D(0, 2) - D(2, 0), z = D(1, 0) - D(0, 1);
+    angle = std::atan2(0.5 * std::sqrt(x * x + y * y + z * z), c);
+  }
+  *angle_deg = angle * (180.0 / M_PI);
   const double d0 = A[3] - B[3], d1 = A[7] - B[7], d2 = A[11] - B[11];
   *trans = std::sqrt(d0 * d0 + d1 * d1 + d2 * d2);
   return GS_OK;
