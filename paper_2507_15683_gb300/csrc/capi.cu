@@ -519,12 +519,14 @@ gs_status enqueue(gs_scene* s, const std::vector<View>& hv, const std::vector<in
   // Early starts of the binning pay where the shading beside it is short: the
   // 1080p render took 264 us without them, 254 us with them; with the pose
   // Jacobian the waiting blocks hold registers that the shading needs (gradient
-  // 634 -> 648 us, visibility check 680 -> 703 us).
-  GS_CUDA(launch_scan_tiles(w, st, !jac));
+  // 634 -> 648 us, visibility check 680 -> 703 us). Kernel timing keeps the
+  // kernels apart.
+  const bool early = !jac && !timed;
+  GS_CUDA(launch_scan_tiles(w, st, early));
   GS_CUDA(mark(3));
-  GS_CUDA(launch_scatter(dviews, w, grid, st, !jac));
+  GS_CUDA(launch_scatter(dviews, w, grid, st, early));
   GS_CUDA(mark(4));
-  GS_CUDA(launch_sort_tiles(w, grid, st, !jac));
+  GS_CUDA(launch_sort_tiles(w, grid, st, early));
   if (!graph) s->counts_zero = true;
   if (fork) GS_CUDA(cudaStreamWaitEvent(st, s->ev_shade, 0));
   GS_CUDA(mark(5));
@@ -554,7 +556,8 @@ gs_status enqueue(gs_scene* s, const std::vector<View>& hv, const std::vector<in
       if (targets_ready) GS_CUDA(cudaStreamWaitEvent(st, targets_ready, 0));  // only this pass reads the targets
       GS_CUDA(launch_composite_tangent(sc, dviews, nv, w, res, cfg, s->sm_count, st));
     }
-    GS_CUDA(launch_reduce_tangent(dviews, nv, w, res, st));
+    // (after bands, the passes in front are on other streams: an ordinary launch behind their events)
+    GS_CUDA(launch_reduce_tangent(dviews, nv, w, res, st, !(bands && bands->n > 0 && nv == 1)));
   }
   GS_CUDA(mark(6));
   if (vis) {

@@ -182,7 +182,8 @@ cudaError_t launch_composite_tangent_range(const SceneDev& sc, const View* views
                                            uint32_t tile_begin, uint32_t tile_end, unsigned int* queue);
 // the fp64 chunk and view sums of the tangent pass's tile partials, once every
 // tile of the call is done
-cudaError_t launch_reduce_tangent(const View* views, int n_views, const Work& w, double* result, cudaStream_t st);
+cudaError_t launch_reduce_tangent(const View* views, int n_views, const Work& w, double* result, cudaStream_t st,
+                                  bool early);
 
 // Algorithm 1 visibility check, after a forward render of one view that wrote
 // final_T and last_idx and a shading pass that wrote the pose Jacobian:

@@ -1027,7 +1027,8 @@ gs_status gs_pnp_solve(gs_pnp* s, const gs_camera* cam, const gs_pose* T_render,
     }
   }
   PNP_CUDA(mark(3));
-  PNP_CUDA(gsr::launch_dependent(early, k_pnp_best, 1, 1024, st, s->counts, n_poses, s->poses64, Tr, s->st));
+  // without a scoring pass in front, an ordinary launch behind the side stream's event
+  PNP_CUDA(gsr::launch_dependent(early && n_hypotheses > 0 && n_matches > 0, k_pnp_best, 1, 1024, st, s->counts, n_poses, s->poses64, Tr, s->st));
   PNP_CUDA(mark(4));
   for (int it = 0; it < opts->refine_iters; ++it) {
     PNP_CUDA(gsr::launch_dependent(early, k_pnp_gn, kGnBlocks, kThreads, st, s->X32, s->nab, s->st, s->partials, fx, fy, tau));

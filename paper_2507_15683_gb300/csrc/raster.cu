@@ -1060,9 +1060,10 @@ cudaError_t launch_composite_tangent(const SceneDev& sc, const View* views, int 
   return cudaGetLastError();
 }
 
-cudaError_t launch_reduce_tangent(const View* views, int n_views, const Work& w, double* result, cudaStream_t st) {
+cudaError_t launch_reduce_tangent(const View* views, int n_views, const Work& w, double* result, cudaStream_t st,
+                                  bool early) {
   if (w.n_tiles == 0 || w.n_chunks == 0) return cudaSuccess;
-  return launch_dependent(true, k_reduce_chunks, (int)w.n_chunks, 7 * 32, st, views, n_views, w, result);
+  return launch_dependent(early, k_reduce_chunks, (int)w.n_chunks, 7 * 32, st, views, n_views, w, result);
 }
 
 cudaError_t launch_composite_tangent_range(const SceneDev& sc, const View* views, int n_views, const Work& w,
