@@ -420,7 +420,8 @@ __global__ void __launch_bounds__(kTileThreads, kProjResident)
       big &= big - 1u;
       const unsigned bn = __shfl_sync(0xffffffffu, n, l), bw = __shfl_sync(0xffffffffu, wd, l);
       const unsigned bf = __shfl_sync(0xffffffffu, first, l), bt = __shfl_sync(0xffffffffu, tx, l);
-      for (unsigned k = lane; k < bn; k += 32u) atomicAdd(&w.tile_ctr[(size_t)(bf + (k / bw) * bt + k % bw) << w.ctr_shift], 1u);
+      for (unsigned k = lane; k < bn; k += 32u)
+        atomicAdd(&w.tile_ctr[(size_t)(bf + (k / bw) * bt + k % bw) << w.ctr_shift], 1u);
     }
   };
   // Gaussian index of flat position f over the active ranges, or -1 (one
@@ -501,205 +502,226 @@ __global__ void __launch_bounds__(kTileThreads, kProjResident)
 }
 
 // Place of d colour_ch / d rho_d in a Jacobian record.
-__host__ __device__ constexpr int jac_colour(int ch, int d) { return d == 2 ? 38 + ch : (ch == 0 ? 10 : ch == 1 ? 34 : 36) + d; }
+__host__ __device__ constexpr int jac_colour(int ch, int d) {
+  return d == 2 ? 38 + ch : (ch == 0 ? 10 : ch == 1 ? 34 : 36) + d;
+}
 
 // ---------------------------------------------------------------------------
 // Shading pass over the compact records: conic, SH colour, float-float
 // blending centre and, for the pose gradient, the per-record pose Jacobian.
 // ---------------------------------------------------------------------------
+constexpr int kShadeSmem = 256 * kJacStride * 4;  // bytes of a gradient's shading block: 44 KB
+static_assert(kShadeSmem <= 48 * 1024, "within the default limit");
+static_assert(kRecRegions % 32 == 0, "a warp's slots are all below the capacity or all above it");
 template <bool GRAD>
 __global__ void __launch_bounds__(256, 3) k_shade(SceneDev sc, const View* __restrict__ views, Work w) {
+  // GRAD: a warp's 32 records leave through shared memory as one contiguous
+  // block (rows of slots without a record hold whatever was there: nothing reads
+  // them): 8 views of 960 x 540 74 us, a 1080p view 24; with each thread storing
+  // its own 176 bytes 94 and 28 us
+  extern __shared__ float4 s_jac[];
+  float4* sj = s_jac + (threadIdx.x >> 5) * (32 * kJacStride / 4);
   if (w.ctr->overflow) return;
   for (uint32_t slot = blockIdx.x * blockDim.x + threadIdx.x; slot < w.rec_cap; slot += gridDim.x * blockDim.x) {
     const uint32_t reg = slot / w.rec_seg, loc = slot - reg * w.rec_seg;
-    if (loc >= min(w.ctr->rec_region[reg].n, w.rec_seg)) continue;
-    const float4 ra = w.rec_a[slot];
-    const int i = __float_as_int(w.rec_b[slot].w);
-    const uint4 m = w.rec_m[slot];
-    const View& V = views[m.z];
-    const float ca = ra.x, cb = ra.y, cc = ra.z;
-    const float4 p4 = __ldg(sc.pos + i);
-    const float4 c0 = __ldg(sc.cov + 2 * i);
-    const float4 c1 = __ldg(sc.cov + 2 * i + 1);
-    const float pz = __uint_as_float(m.w);
-    // conic from the binary32 covariance; determinant with one compensated step
-    const float bb = cb * cb;
-    const float e = __fmaf_rn(-cb, cb, bb);
-    const float f = __fmaf_rn(ca, cc, -bb);
-    const float detc = f + e;
-    const float inv = 1.0f / detc;
-    const float A = cc * inv, B = -cb * inv, C = ca * inv;
-    // colour from SH at dir = normalize(mean - camera centre)
-    const float dxw = p4.x - V.cw[0], dyw = p4.y - V.cw[1], dzw = p4.z - V.cw[2];
-    const float dn = sqrtf(dxw * dxw + dyw * dyw + dzw * dzw);
-    const float rn = 1.0f / dn;
-    const float dirx = dxw * rn, diry = dyw * rn, dirz = dzw * rn;
-    float rgb[3], G[3][3];
-    eval_sh_deg<GRAD>(sc.sh_degree, sc.sh + (size_t)i * sc.nsh4, dirx, diry, dirz, rgb, G);
-    bool clampc[3];
+    const bool filled = loc < min(w.ctr->rec_region[reg].n, w.rec_seg);
+    if (GRAD ? !__any_sync(0xffffffffu, filled) : !filled) continue;
+    if (filled) {
+      const float4 ra = w.rec_a[slot];
+      const int i = __float_as_int(w.rec_b[slot].w);
+      const uint4 m = w.rec_m[slot];
+      const View& V = views[m.z];
+      const float ca = ra.x, cb = ra.y, cc = ra.z;
+      const float4 p4 = __ldg(sc.pos + i);
+      const float4 c0 = __ldg(sc.cov + 2 * i);
+      const float4 c1 = __ldg(sc.cov + 2 * i + 1);
+      const float pz = __uint_as_float(m.w);
+      // conic from the binary32 covariance; determinant with one compensated step
+      const float bb = cb * cb;
+      const float e = __fmaf_rn(-cb, cb, bb);
+      const float f = __fmaf_rn(ca, cc, -bb);
+      const float detc = f + e;
+      const float inv = 1.0f / detc;
+      const float A = cc * inv, B = -cb * inv, C = ca * inv;
+      // colour from SH at dir = normalize(mean - camera centre)
+      const float dxw = p4.x - V.cw[0], dyw = p4.y - V.cw[1], dzw = p4.z - V.cw[2];
+      const float dn = sqrtf(dxw * dxw + dyw * dyw + dzw * dzw);
+      const float rn = 1.0f / dn;
+      const float dirx = dxw * rn, diry = dyw * rn, dirz = dzw * rn;
+      float rgb[3], G[3][3];
+      eval_sh_deg<GRAD>(sc.sh_degree, sc.sh + (size_t)i * sc.nsh4, dirx, diry, dirz, rgb, G);
+      bool clampc[3];
 #pragma unroll
-    for (int ch = 0; ch < 3; ++ch) {
-      clampc[ch] = rgb[ch] < 0.0f;
-      rgb[ch] = fmaxf(rgb[ch], 0.0f);
-    }
-    // blending centre in float-float; high parts in rec_a, low parts as half2
-    const ff fpx = ff_row(V.R, V.Rl, V.t[0], V.tl[0], p4.x, p4.y, p4.z);
-    const ff fpy = ff_row(V.R + 3, V.Rl + 3, V.t[1], V.tl[1], p4.x, p4.y, p4.z);
-    const ff fpz = ff_row(V.R + 6, V.Rl + 6, V.t[2], V.tl[2], p4.x, p4.y, p4.z);
-    const ff fu = ff_project(fpx, fpz, V.fx, V.cx);
-    const ff fv = ff_project(fpy, fpz, V.fy, V.cy);
-    const __half2 lo2 = __floats2half2_rn(fu.lo, fv.lo);
-    w.rec_a[slot] = make_float4(fu.hi, fv.hi, A, B);
-    // rec_b.w (the Gaussian index, the sort's tie key) stays as the projection wrote it
-    float* rb = reinterpret_cast<float*>(w.rec_b + slot);
-    *reinterpret_cast<float2*>(rb) = make_float2(C, c1.z);
-    rb[2] = pz;
-    w.rec_c[slot] = make_float4(rgb[0], rgb[1], rgb[2], *reinterpret_cast<const float*>(&lo2));
+      for (int ch = 0; ch < 3; ++ch) {
+        clampc[ch] = rgb[ch] < 0.0f;
+        rgb[ch] = fmaxf(rgb[ch], 0.0f);
+      }
+      // blending centre in float-float; high parts in rec_a, low parts as half2
+      const ff fpx = ff_row(V.R, V.Rl, V.t[0], V.tl[0], p4.x, p4.y, p4.z);
+      const ff fpy = ff_row(V.R + 3, V.Rl + 3, V.t[1], V.tl[1], p4.x, p4.y, p4.z);
+      const ff fpz = ff_row(V.R + 6, V.Rl + 6, V.t[2], V.tl[2], p4.x, p4.y, p4.z);
+      const ff fu = ff_project(fpx, fpz, V.fx, V.cx);
+      const ff fv = ff_project(fpy, fpz, V.fy, V.cy);
+      const __half2 lo2 = __floats2half2_rn(fu.lo, fv.lo);
+      w.rec_a[slot] = make_float4(fu.hi, fv.hi, A, B);
+      // rec_b.w (the Gaussian index, the sort's tie key) stays as the projection wrote it
+      float* rb = reinterpret_cast<float*>(w.rec_b + slot);
+      *reinterpret_cast<float2*>(rb) = make_float2(C, c1.z);
+      rb[2] = pz;
+      w.rec_c[slot] = make_float4(rgb[0], rgb[1], rgb[2], *reinterpret_cast<const float*>(&lo2));
 
-    if (GRAD) {
-      // Pose Jacobian of (u, v, A, B, C, z) w.r.t. xi = (rho, phi) and of (r, g, b)
-      // w.r.t. rho, by forward differentiation along the six tangent directions:
-      // d p = rho + phi x p; d Sigma_cam = [phi]x Sigma_cam - Sigma_cam [phi]x;
-      // d (mean - camera centre) = R^T rho.
-      const float* R = V.R;
-      const float px = fpx.hi, py = fpy.hi;
-      const float ix = px / pz, iy = py / pz;
-      const float Sw[3][3] = {{c0.x, c0.y, c0.z}, {c0.y, c0.w, c1.x}, {c0.z, c1.x, c1.y}};
-      float Q[3][3], Sc[3][3];
+      if (GRAD) {
+        // Pose Jacobian of (u, v, A, B, C, z) w.r.t. xi = (rho, phi) and of (r, g, b)
+        // w.r.t. rho, by forward differentiation along the six tangent directions:
+        // d p = rho + phi x p; d Sigma_cam = [phi]x Sigma_cam - Sigma_cam [phi]x;
+        // d (mean - camera centre) = R^T rho.
+        const float* R = V.R;
+        const float px = fpx.hi, py = fpy.hi;
+        const float ix = px / pz, iy = py / pz;
+        const float Sw[3][3] = {{c0.x, c0.y, c0.z}, {c0.y, c0.w, c1.x}, {c0.z, c1.x, c1.y}};
+        float Q[3][3], Sc[3][3];
 #pragma unroll
-      for (int a = 0; a < 3; ++a)
+        for (int a = 0; a < 3; ++a)
 #pragma unroll
-        for (int b = 0; b < 3; ++b) Q[a][b] = R[3 * a] * Sw[0][b] + R[3 * a + 1] * Sw[1][b] + R[3 * a + 2] * Sw[2][b];
+          for (int b = 0; b < 3; ++b) Q[a][b] = R[3 * a] * Sw[0][b] + R[3 * a + 1] * Sw[1][b] + R[3 * a + 2] * Sw[2][b];
 #pragma unroll
-      for (int a = 0; a < 3; ++a)
+        for (int a = 0; a < 3; ++a)
 #pragma unroll
-        for (int b = 0; b < 3; ++b) Sc[a][b] = Q[a][0] * R[3 * b] + Q[a][1] * R[3 * b + 1] + Q[a][2] * R[3 * b + 2];
-      const bool clx = (ix < -V.limx) || (ix > V.limx);
-      const bool cly = (iy < -V.limy) || (iy > V.limy);
-      const float Lx = ix < 0.0f ? -V.limx : V.limx, Ly = iy < 0.0f ? -V.limy : V.limy;
-      const float zi = 1.0f / pz;
-      const float xh = clx ? Lx * pz : px, yh = cly ? Ly * pz : py;
-      const float j00 = V.fx * zi, j02 = -V.fx * xh * zi * zi;
-      const float j11 = V.fy * zi, j12 = -V.fy * yh * zi * zi;
-      float K[2][3];
+          for (int b = 0; b < 3; ++b) Sc[a][b] = Q[a][0] * R[3 * b] + Q[a][1] * R[3 * b + 1] + Q[a][2] * R[3 * b + 2];
+        const bool clx = (ix < -V.limx) || (ix > V.limx);
+        const bool cly = (iy < -V.limy) || (iy > V.limy);
+        const float Lx = ix < 0.0f ? -V.limx : V.limx, Ly = iy < 0.0f ? -V.limy : V.limy;
+        const float zi = 1.0f / pz;
+        const float xh = clx ? Lx * pz : px, yh = cly ? Ly * pz : py;
+        const float j00 = V.fx * zi, j02 = -V.fx * xh * zi * zi;
+        const float j11 = V.fy * zi, j12 = -V.fy * yh * zi * zi;
+        float K[2][3];
 #pragma unroll
-      for (int k = 0; k < 3; ++k) {
-        K[0][k] = j00 * Sc[0][k] + j02 * Sc[2][k];
-        K[1][k] = j11 * Sc[1][k] + j12 * Sc[2][k];
-      }
-      const float di = 1.0f / detc;
-      float jac[45];
-      const float pc[3] = {px, py, pz};
-#pragma unroll
-      for (int k = 0; k < 6; ++k) {
-        float dp[3];
-        if (k < 3) {
-          dp[0] = (k == 0) ? 1.f : 0.f;
-          dp[1] = (k == 1) ? 1.f : 0.f;
-          dp[2] = (k == 2) ? 1.f : 0.f;
-        } else {
-          const int e3 = k - 3;  // e x p
-          dp[0] = (e3 == 1) ? pc[2] : (e3 == 2) ? -pc[1] : 0.f;
-          dp[1] = (e3 == 0) ? -pc[2] : (e3 == 2) ? pc[0] : 0.f;
-          dp[2] = (e3 == 0) ? pc[1] : (e3 == 1) ? -pc[0] : 0.f;
+        for (int k = 0; k < 3; ++k) {
+          K[0][k] = j00 * Sc[0][k] + j02 * Sc[2][k];
+          K[1][k] = j11 * Sc[1][k] + j12 * Sc[2][k];
         }
-        const float du = V.fx * (dp[0] - ix * dp[2]) * zi;
-        const float dv = V.fy * (dp[1] - iy * dp[2]) * zi;
-        const float dxh = clx ? Lx * dp[2] : dp[0];
-        const float dyh = cly ? Ly * dp[2] : dp[1];
-        const float dj00 = -j00 * dp[2] * zi;
-        const float dj02 = -V.fx * (dxh - 2.0f * xh * dp[2] * zi) * zi * zi;
-        const float dj11 = -j11 * dp[2] * zi;
-        const float dj12 = -V.fy * (dyh - 2.0f * yh * dp[2] * zi) * zi * zi;
-        // S = dJ K^T
-        const float S00 = dj00 * K[0][0] + dj02 * K[0][2];
-        const float S01 = dj00 * K[1][0] + dj02 * K[1][2];
-        const float S10 = dj11 * K[0][1] + dj12 * K[0][2];
-        const float S11 = dj11 * K[1][1] + dj12 * K[1][2];
-        float dm00 = 2.0f * S00, dm01 = S01 + S10, dm11 = 2.0f * S11;
-        if (k >= 3) {
-          // D = X + X^T with X = [e]x Sc
-          const int e3 = k - 3;
-          float X[3][3];
+        const float di = 1.0f / detc;
+        float jac[45];
+        const float pc[3] = {px, py, pz};
 #pragma unroll
-          for (int b = 0; b < 3; ++b) {
-            if (e3 == 0) { X[0][b] = 0.f; X[1][b] = -Sc[2][b]; X[2][b] = Sc[1][b]; }
-            else if (e3 == 1) { X[0][b] = Sc[2][b]; X[1][b] = 0.f; X[2][b] = -Sc[0][b]; }
-            else { X[0][b] = -Sc[1][b]; X[1][b] = Sc[0][b]; X[2][b] = 0.f; }
+        for (int k = 0; k < 6; ++k) {
+          float dp[3];
+          if (k < 3) {
+            dp[0] = (k == 0) ? 1.f : 0.f;
+            dp[1] = (k == 1) ? 1.f : 0.f;
+            dp[2] = (k == 2) ? 1.f : 0.f;
+          } else {
+            const int e3 = k - 3;  // e x p
+            dp[0] = (e3 == 1) ? pc[2] : (e3 == 2) ? -pc[1] : 0.f;
+            dp[1] = (e3 == 0) ? -pc[2] : (e3 == 2) ? pc[0] : 0.f;
+            dp[2] = (e3 == 0) ? pc[1] : (e3 == 1) ? -pc[0] : 0.f;
           }
-          float D[3][3];
+          const float du = V.fx * (dp[0] - ix * dp[2]) * zi;
+          const float dv = V.fy * (dp[1] - iy * dp[2]) * zi;
+          const float dxh = clx ? Lx * dp[2] : dp[0];
+          const float dyh = cly ? Ly * dp[2] : dp[1];
+          const float dj00 = -j00 * dp[2] * zi;
+          const float dj02 = -V.fx * (dxh - 2.0f * xh * dp[2] * zi) * zi * zi;
+          const float dj11 = -j11 * dp[2] * zi;
+          const float dj12 = -V.fy * (dyh - 2.0f * yh * dp[2] * zi) * zi * zi;
+          // S = dJ K^T
+          const float S00 = dj00 * K[0][0] + dj02 * K[0][2];
+          const float S01 = dj00 * K[1][0] + dj02 * K[1][2];
+          const float S10 = dj11 * K[0][1] + dj12 * K[0][2];
+          const float S11 = dj11 * K[1][1] + dj12 * K[1][2];
+          float dm00 = 2.0f * S00, dm01 = S01 + S10, dm11 = 2.0f * S11;
+          if (k >= 3) {
+            // D = X + X^T with X = [e]x Sc
+            const int e3 = k - 3;
+            float X[3][3];
 #pragma unroll
-          for (int a = 0; a < 3; ++a)
+            for (int b = 0; b < 3; ++b) {
+              if (e3 == 0) { X[0][b] = 0.f; X[1][b] = -Sc[2][b]; X[2][b] = Sc[1][b]; }
+              else if (e3 == 1) { X[0][b] = Sc[2][b]; X[1][b] = 0.f; X[2][b] = -Sc[0][b]; }
+              else { X[0][b] = -Sc[1][b]; X[1][b] = Sc[0][b]; X[2][b] = 0.f; }
+            }
+            float D[3][3];
 #pragma unroll
-            for (int b = 0; b < 3; ++b) D[a][b] = X[a][b] + X[b][a];
-          float JD[2][3];
+            for (int a = 0; a < 3; ++a)
 #pragma unroll
-          for (int b = 0; b < 3; ++b) {
-            JD[0][b] = j00 * D[0][b] + j02 * D[2][b];
-            JD[1][b] = j11 * D[1][b] + j12 * D[2][b];
+              for (int b = 0; b < 3; ++b) D[a][b] = X[a][b] + X[b][a];
+            float JD[2][3];
+#pragma unroll
+            for (int b = 0; b < 3; ++b) {
+              JD[0][b] = j00 * D[0][b] + j02 * D[2][b];
+              JD[1][b] = j11 * D[1][b] + j12 * D[2][b];
+            }
+            dm00 += JD[0][0] * j00 + JD[0][2] * j02;
+            dm01 += JD[0][1] * j11 + JD[0][2] * j12;
+            dm11 += JD[1][1] * j11 + JD[1][2] * j12;
           }
-          dm00 += JD[0][0] * j00 + JD[0][2] * j02;
-          dm01 += JD[0][1] * j11 + JD[0][2] * j12;
-          dm11 += JD[1][1] * j11 + JD[1][2] * j12;
+          const float ddet = dm00 * cc + ca * dm11 - 2.0f * cb * dm01;
+          const float dA = (dm11 - cc * ddet * di) * di;
+          const float dB = -(dm01 - cb * ddet * di) * di;
+          const float dC = (dm00 - ca * ddet * di) * di;
+          jac[0 * 6 + k] = du;
+          jac[1 * 6 + k] = dv;
+          jac[2 * 6 + k] = dA;
+          jac[3 * 6 + k] = dB;
+          jac[4 * 6 + k] = dC;
+          jac[5 * 6 + k] = dp[2];
         }
-        const float ddet = dm00 * cc + ca * dm11 - 2.0f * cb * dm01;
-        const float dA = (dm11 - cc * ddet * di) * di;
-        const float dB = -(dm01 - cb * ddet * di) * di;
-        const float dC = (dm00 - ca * ddet * di) * di;
-        jac[0 * 6 + k] = du;
-        jac[1 * 6 + k] = dv;
-        jac[2 * 6 + k] = dA;
-        jac[3 * 6 + k] = dB;
-        jac[4 * 6 + k] = dC;
-        jac[5 * 6 + k] = dp[2];
-      }
-      // colour rows (rho only): d rgb_ch / d rho_k = G_ch . (I - dir dir^T) R^T e_k / |d|
+        // colour rows (rho only): d rgb_ch / d rho_k = G_ch . (I - dir dir^T) R^T e_k / |d|
 #pragma unroll
-      for (int ch = 0; ch < 3; ++ch) {
-        const float gd = G[ch][0] * dirx + G[ch][1] * diry + G[ch][2] * dirz;
-        const float gp0 = (G[ch][0] - gd * dirx) * rn, gp1 = (G[ch][1] - gd * diry) * rn,
-                    gp2 = (G[ch][2] - gd * dirz) * rn;
+        for (int ch = 0; ch < 3; ++ch) {
+          const float gd = G[ch][0] * dirx + G[ch][1] * diry + G[ch][2] * dirz;
+          const float gp0 = (G[ch][0] - gd * dirx) * rn, gp1 = (G[ch][1] - gd * diry) * rn,
+                      gp2 = (G[ch][2] - gd * dirz) * rn;
 #pragma unroll
-        for (int k = 0; k < 3; ++k)
-          jac[36 + 3 * ch + k] = clampc[ch] ? 0.0f : gp0 * R[3 * k] + gp1 * R[3 * k + 1] + gp2 * R[3 * k + 2];
-      }
-      // Stored for the compositor's packed FMAs over the direction pairs
-      // (0,1), (2,3), (4,5). With the pixel offset (dx, dy) = centre - pixel,
-      //   -dpower/dxi = dx (A du + B dv) + dy (B du + C dv) + dx^2 dA/2
-      //                 + dx dy dB + dy^2 dC/2,
-      // so pair k holds (P, Q), (dA/2, dB) and dC/2, each as the two
-      // directions of the pair, with P = A du + B dv and Q = B du + C dv, in
-      // two and a half float4. The other halves hold d(r, g)/d rho_0..1 and
-      // the two entries of dz that are not 0 or 1 (dz/dphi_0 = py,
-      // dz/dphi_1 = -px), and two more float4 the rest of the colour rows and
-      // the colour: 11 float4, every word used. With dz in full, zeros behind
-      // the colour rows and the colour apart it was 12 and the tangent pass
-      // read 15 vectors per hit, not 13: the shading pass of 8 views of
-      // 960 x 540 took 111 us, now 93; the tangent pass takes the same time.
-      float jt[kJacStride];
-#pragma unroll
-      for (int k = 0; k < 3; ++k) {
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          const int d = 2 * k + h;
-          jt[12 * k + h] = A * jac[d] + B * jac[6 + d];
-          jt[12 * k + 2 + h] = B * jac[d] + C * jac[6 + d];
-          jt[12 * k + 4 + h] = 0.5f * jac[12 + d];
-          jt[12 * k + 6 + h] = jac[18 + d];
-          jt[12 * k + 8 + h] = 0.5f * jac[24 + d];
+          for (int k = 0; k < 3; ++k)
+            jac[36 + 3 * ch + k] = clampc[ch] ? 0.0f : gp0 * R[3 * k] + gp1 * R[3 * k + 1] + gp2 * R[3 * k + 2];
         }
+        // Stored for the compositor's packed FMAs over the direction pairs
+        // (0,1), (2,3), (4,5). With the pixel offset (dx, dy) = centre - pixel,
+        //   -dpower/dxi = dx (A du + B dv) + dy (B du + C dv) + dx^2 dA/2
+        //                 + dx dy dB + dy^2 dC/2,
+        // so pair k holds (P, Q), (dA/2, dB) and dC/2, each as the two
+        // directions of the pair, with P = A du + B dv and Q = B du + C dv, in
+        // two and a half float4. The other halves hold d(r, g)/d rho_0..1 and
+        // the two entries of dz that are not 0 or 1 (dz/dphi_0 = py,
+        // dz/dphi_1 = -px), and two more float4 the rest of the colour rows and
+        // the colour: 11 float4, every word used. With dz in full, zeros behind
+        // the colour rows and the colour apart it was 12 and the tangent pass
+        // read 15 vectors per hit, not 13: the shading pass of 8 views of
+        // 960 x 540 took 111 us, then 93; the tangent pass takes the same time.
+        float jt[kJacStride];
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            const int d = 2 * k + h;
+            jt[12 * k + h] = A * jac[d] + B * jac[6 + d];
+            jt[12 * k + 2 + h] = B * jac[d] + C * jac[6 + d];
+            jt[12 * k + 4 + h] = 0.5f * jac[12 + d];
+            jt[12 * k + 6 + h] = jac[18 + d];
+            jt[12 * k + 8 + h] = 0.5f * jac[24 + d];
+          }
+        }
+        jt[22] = jac[33];  // dz/dphi_0, dz/dphi_1
+        jt[23] = jac[34];
+#pragma unroll
+        for (int ch = 0; ch < 3; ++ch) {
+#pragma unroll
+          for (int k = 0; k < 3; ++k) jt[jac_colour(ch, k)] = jac[36 + 3 * ch + k];
+          jt[41 + ch] = rgb[ch];
+        }
+        float4* jo = sj + (threadIdx.x & 31) * (kJacStride / 4);
+#pragma unroll
+        for (int q = 0; q < kJacStride / 4; ++q) jo[q] = make_float4(jt[4 * q], jt[4 * q + 1], jt[4 * q + 2], jt[4 * q + 3]);
       }
-      jt[22] = jac[33];  // dz/dphi_0, dz/dphi_1
-      jt[23] = jac[34];
+    }
+    if (GRAD) {  // rec_cap is a multiple of 64: the warp's slots are all below it
+      __syncwarp();
+      float4* out = reinterpret_cast<float4*>(w.rec_j + (size_t)(slot & ~31u) * kJacStride);
 #pragma unroll
-      for (int ch = 0; ch < 3; ++ch) {
-#pragma unroll
-        for (int k = 0; k < 3; ++k) jt[jac_colour(ch, k)] = jac[36 + 3 * ch + k];
-        jt[41 + ch] = rgb[ch];
-      }
-      float4* jo = reinterpret_cast<float4*>(w.rec_j + (size_t)slot * kJacStride);
-#pragma unroll
-      for (int q = 0; q < kJacStride / 4; ++q) jo[q] = make_float4(jt[4 * q], jt[4 * q + 1], jt[4 * q + 2], jt[4 * q + 3]);
+      for (int q = 0; q < kJacStride / 4; ++q) out[q * 32 + (threadIdx.x & 31)] = sj[q * 32 + (threadIdx.x & 31)];
+      __syncwarp();  // before the next records' rows
     }
   }
 }
@@ -904,7 +926,7 @@ cudaError_t launch_shade(const SceneDev& sc, const View* views, const Work& w, b
   const int need = (int)((w.rec_cap + 255) / 256);
   const int g = need < grid ? need : grid;
   if (grad)
-    k_shade<true><<<g, 256, 0, st>>>(sc, views, w);
+    k_shade<true><<<g, 256, kShadeSmem, st>>>(sc, views, w);
   else
     k_shade<false><<<g, 256, 0, st>>>(sc, views, w);
   return cudaGetLastError();
