@@ -809,7 +809,8 @@ gs_status run_graph(gs_scene* s, GraphCache& G, const std::vector<char>& key, co
   const int n_views = (int)hv.size();
   std::vector<int4> ranges;
   const bool ready = G.valid && G.key == key && G.gen == g_alloc_gen.load();
-  if (ready) GS_CUDA(cudaEventSynchronize(G.done));  // previous replay read the table
+  // the last replay has read the table, which is overwritten below, or freed for a new capture's
+  if (G.exec) GS_CUDA(cudaEventSynchronize(G.done));
   GS_TRY(prepare_call(s, hv, st, ranges));  // uploads partitions on st before the graph runs
   if (!ready) {
     if (G.exec) cudaGraphExecDestroy(G.exec);
