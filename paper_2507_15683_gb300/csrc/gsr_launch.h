@@ -1,8 +1,34 @@
-// Early starts of dependent kernels (programmatic stream serialization).
+// Early starts of dependent kernels (programmatic stream serialization), and
+// launch parameters that belong to a device.
 #pragma once
 #include <cuda_runtime.h>
 
+#include <atomic>
+
 namespace gsr {
+
+// A positive number per device, made at the first use there. cudaFuncSetAttribute
+// and the occupancy queries act on the current device, so what they set or return
+// is not another device's. Threads whose first uses coincide each make it, and
+// store the same.
+class PerDevice {
+ public:
+  template <typename F>
+  int get(F make) {
+    int dev = -1;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kDevices) return make();
+    int x = v_[dev].load(std::memory_order_acquire);
+    if (x == 0) {
+      x = make();
+      v_[dev].store(x, std::memory_order_release);
+    }
+    return x;
+  }
+
+ private:
+  static constexpr int kDevices = 64;  // above: made at every use
+  std::atomic<int> v_[kDevices] = {};
+};
 
 // A kernel launched by launch_dependent may start (its blocks become resident)
 // before the kernel in front of it on the stream has ended, once all blocks of

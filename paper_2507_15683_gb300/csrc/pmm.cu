@@ -1337,6 +1337,11 @@ gs_status gs_pmm_create(int channels, int height, int width, gs_pmm** out) {
   m->nb = (n + kTile - 1) / kTile;
   cudaError_t e = cudaGetDevice(&m->device);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&m->sm_count, cudaDevAttrMultiProcessorCount, m->device);
+  // the tile passes' shared memory, on this matcher's device
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(k_pmm_sums, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSumSmemBytes);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(k_pmm_argmax, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBestSmemBytes);
   // pass 2: two CTAs per SM, equal runs of tiles
   const int tiles = m->nb * m->nb, ctas = std::min(tiles, 2 * m->sm_count);
   m->per = (tiles + ctas - 1) / ctas;
@@ -1444,12 +1449,6 @@ gs_status gs_pmm_match(gs_pmm* m, const float* feat_query, const float* feat_ren
   const CodeMap mr{feat_render, reinterpret_cast<unsigned short*>(m->codes_r), m->tiled_r, nullptr};
   k_pmm_codes<<<cgrid, 1024, 0, st>>>(mq, mr, m->H, m->W, m->Wc);
   PMM_CUDA(cudaGetLastError());
-  static bool attr = false;
-  if (!attr) {
-    PMM_CUDA(cudaFuncSetAttribute(k_pmm_sums, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSumSmemBytes));
-    PMM_CUDA(cudaFuncSetAttribute(k_pmm_argmax, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBestSmemBytes));
-    attr = true;
-  }
   const int tiles = nb * nb;
   const unsigned char* cq = m->tiled_q;
   const unsigned char* cr = m->tiled_r;

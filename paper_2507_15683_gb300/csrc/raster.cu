@@ -991,17 +991,17 @@ const Variant* variant_table(int mode) {
   return mode == kModeTan ? tan : mode == kModeFwdFeat ? feat : fwd;
 }
 
-// resident CTAs per SM of a variant (its shared memory and registers), once per process
+// resident CTAs per SM of a variant (its shared memory and registers) on the current device; also lets the
+// variant have its shared memory there
 int variant_occupancy(int mode, int v) {
-  static int occ[kModeCount][kCompVariants] = {};
-  if (occ[mode][v] == 0) {
+  static PerDevice occ[kModeCount][kCompVariants];
+  return occ[mode][v].get([&] {
     const Variant& V = variant_table(mode)[v];
     cudaFuncSetAttribute(V.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, V.smem);
     int b = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, V.fn, kTileThreads, V.smem) != cudaSuccess || b < 1) b = 1;
-    occ[mode][v] = b;
-  }
-  return occ[mode][v];
+    return b;
+  });
 }
 
 int clamp_variant(int v) { return v >= 0 && v < kCompVariants ? v : 0; }
@@ -1037,14 +1037,13 @@ cudaError_t launch_composite(const SceneDev& sc, const View* views, int n_views,
 cudaError_t launch_vis_backward(const View* views, int n_views, const Work& w, float* acc, int sm_count,
                                 cudaStream_t st) {
   if (w.n_tiles == 0) return cudaSuccess;
-  static int per_sm = 0;  // resident blocks per SM (persistent grid)
-  if (per_sm == 0) {
+  static PerDevice per_sm;  // resident blocks per SM (persistent grid)
+  const int grid = sm_count * per_sm.get([] {
     int b = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_vis_backward, kTileThreads, 0) != cudaSuccess || b < 1)
       b = 4;
-    per_sm = b;
-  }
-  const int grid = sm_count * per_sm;
+    return b;
+  });
   const int g = (uint32_t)grid < w.n_tiles ? grid : (int)w.n_tiles;
   k_vis_backward<<<g, kTileThreads, 0, st>>>(views, n_views, w, acc);
   return cudaGetLastError();

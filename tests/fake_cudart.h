@@ -47,6 +47,7 @@ inline std::vector<std::string> violations;
 inline std::map<int, int> occupancy = {{0, 4}, {1, 3}};
 inline Stream legacy;
 inline thread_local int device = 0;
+inline thread_local cudaError_t last_error = cudaSuccess;
 inline thread_local cudaStreamCaptureMode mode = cudaStreamCaptureModeGlobal;
 inline bool other_capture = false;  // another thread captures in global mode
 
@@ -89,9 +90,10 @@ inline cudaError_t put(cudaStream_t s, Op o) {
   queue.push_back(std::move(o));
   return cudaSuccess;
 }
-inline cudaError_t launch(const void* f, size_t smem, cudaStream_t s, bool early) {
+inline cudaError_t launch(const void* f, dim3 grid, size_t smem, cudaStream_t s, bool early) {
   count["kernel " + names[f]]++;
-  if (smem > 48 * 1024 && !large_smem.count({device, f})) return cudaErrorInvalidValue;
+  count["grid " + names[f]] = (int)grid.x;
+  if (smem > 48 * 1024 && !large_smem.count({device, f})) return last_error = cudaErrorInvalidValue;
   if (early && of(s)->last != kKernel) violate(names[f] + " may start early but no kernel is in front of it");
   Op o;
   o.kind = kKernel;
@@ -111,7 +113,8 @@ void __cudaRegisterFatBinaryEnd(void**) {}
 void __cudaUnregisterFatBinary(void**) {}
 void __cudaRegisterFunction(void**, const char* f, char*, const char* name, int, uint3*, uint3*, dim3*, dim3*, int*) {
   std::string s = name;  // mangled: the identifier is enough
-  for (const char* k : {"k_project", "k_scan_tiles", "k_refine_update", "k_pnp_scan", "k_pmm_sums", "k_composite"})
+  for (const char* k : {"k_project", "k_scan_tiles", "k_refine_update", "k_pnp_scan", "k_pmm_sums", "k_composite",
+                        "k_vis_backward"})
     if (s.find(k) != std::string::npos) s = k;
   fake::names[f] = s;
 }
@@ -134,15 +137,15 @@ cudaError_t __cudaGetKernel(cudaKernel_t* k, const void* f) {
   *k = (cudaKernel_t)f;
   return cudaSuccess;
 }
-cudaError_t __cudaLaunchKernel(cudaKernel_t k, dim3, dim3, void**, size_t smem, cudaStream_t s) {
-  return fake::launch((const void*)k, smem, s, false);
+cudaError_t __cudaLaunchKernel(cudaKernel_t k, dim3 grid, dim3, void**, size_t smem, cudaStream_t s) {
+  return fake::launch((const void*)k, grid, smem, s, false);
 }
 cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t* c, const void* f, void**) {
   bool early = false;
   for (unsigned i = 0; i < c->numAttrs; ++i)
     early = early || (c->attrs[i].id == cudaLaunchAttributeProgrammaticStreamSerialization &&
                       c->attrs[i].val.programmaticStreamSerializationAllowed);
-  return fake::launch(f, c->dynamicSmemBytes, c->stream, early);
+  return fake::launch(f, c->gridDim, c->dynamicSmemBytes, c->stream, early);
 }
 cudaError_t cudaFuncSetAttribute(const void* f, cudaFuncAttribute, int) {
   fake::large_smem.insert({fake::device, f});
@@ -172,7 +175,11 @@ cudaError_t cudaGetDeviceProperties(cudaDeviceProp* p, int) {
   p->multiProcessorCount = 152;
   return cudaSuccess;
 }
-cudaError_t cudaGetLastError() { return cudaSuccess; }
+cudaError_t cudaGetLastError() {
+  const cudaError_t e = fake::last_error;
+  fake::last_error = cudaSuccess;
+  return e;
+}
 const char* cudaGetErrorString(cudaError_t e) {
   static thread_local char s[32];
   std::snprintf(s, sizeof(s), "error %d", (int)e);

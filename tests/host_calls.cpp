@@ -3,6 +3,7 @@
 #include "fake_cudart.h"
 
 #include "gsr.h"
+#include "gsr_pmm.h"
 
 static int failed = 0;
 #define CHECK(x)                                                \
@@ -28,10 +29,12 @@ static gs_pose pose(double z) {
   p.T_cw[11] = z;
   return p;
 }
-static gs_scene* scene(int64_t n) {
+static gs_scene* scene(int64_t n, int feat_dim = 0) {
   static std::vector<float> v(4096, 0.5f);
   gs_scene_desc d{};
   d.n = n;
+  d.feat_dim = feat_dim;
+  d.feats_bf16 = feat_dim ? (const uint16_t*)v.data() : nullptr;
   d.means = d.scales = d.quats = d.opacities = d.sh = v.data();
   d.device_resident = 1;
   gs_scene* s = nullptr;
@@ -53,8 +56,34 @@ static void batches_of_changing_size() {
   gs_destroy_scene(s);
 }
 
+// A second device of the process: kernels with large shared memory are allowed it
+// there too, and the persistent grids are that device's.
+static void two_devices() {
+  static float maps[2][32 * 64 * 64] __attribute__((aligned(16))), image[32 * 256 * 256];
+  for (int d = 0; d < 2; ++d) {
+    cudaSetDevice(d);
+    gs_scene* s = scene(100, 32);
+    gs_outputs o{};
+    o.feats = image;
+    const gs_camera c = camera(1920, 1080);
+    const gs_pose p = pose(0);
+    CHECK(gs_render(s, &c, &p, &o, nullptr) == GS_OK);
+    CHECK(fake::count["grid k_composite"] == 152 * fake::occupancy[d]);
+    std::vector<uint8_t> mask(100);
+    CHECK(gs_visibility(s, &c, &p, mask.data(), nullptr, nullptr, nullptr, nullptr, nullptr, nullptr) == GS_OK);
+    CHECK(fake::count["grid k_vis_backward"] == 152 * fake::occupancy[d]);
+    gs_destroy_scene(s);
+    gs_pmm* m = nullptr;
+    CHECK(gs_pmm_create(32, 64, 64, &m) == GS_OK);
+    gs_pmm_result r{};
+    CHECK(gs_pmm_match(m, maps[0], maps[1], 0.1f, &r, nullptr) == GS_OK);
+    gs_pmm_destroy(m);
+  }
+}
+
 int main(int argc, char** argv) {
-  const std::map<std::string, void (*)()> all = {{"batches_of_changing_size", batches_of_changing_size}};
+  const std::map<std::string, void (*)()> all = {{"batches_of_changing_size", batches_of_changing_size},
+                                                    {"two_devices", two_devices}};
   const auto it = all.find(argc > 1 ? argv[1] : "");
   if (it == all.end()) return 2;
   it->second();
