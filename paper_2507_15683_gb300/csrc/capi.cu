@@ -520,8 +520,9 @@ gs_status enqueue(gs_scene* s, const std::vector<View>& hv, const std::vector<in
   // 1080p render took 264 us without them, 254 us with them; with the pose
   // Jacobian the waiting blocks hold registers that the shading needs (gradient
   // 634 -> 648 us, visibility check 680 -> 703 us). Kernel timing keeps the
-  // kernels apart.
-  const bool early = !jac && !timed;
+  // kernels apart. Without a Gaussian there is no projection or shading, and so
+  // no kernel that the scan could start behind.
+  const bool early = !jac && !timed && s->n > 0;
   GS_CUDA(launch_scan_tiles(w, st, early));
   GS_CUDA(mark(3));
   GS_CUDA(launch_scatter(dviews, w, grid, st, early));
@@ -2023,10 +2024,11 @@ gs_status refine_on_device(gs_scene* s, int nv, const gs_camera* cams, gs_pose* 
   }
   const int blocks = (nv + 3) / 4;
   gs_status status = GS_OK;
-  auto launch_update = [&](cudaStream_t on) -> gs_status {
+  // early: directly behind the reduction of the iteration's partials
+  auto launch_update = [&](cudaStream_t on, bool early) -> gs_status {
     View* dviews = reinterpret_cast<View*>(static_cast<char*>(s->views.p) + table_views_off(s));
-    GS_CUDA(launch_dependent(true, k_refine_update, blocks, 128, on, dviews, nv, dp<double>(s->result), drs, *o, iters, dhist,
-                             dp<Counters>(s->views), dsticky));
+    GS_CUDA(launch_dependent(early, k_refine_update, blocks, 128, on, dviews, nv, dp<double>(s->result), drs, *o, iters,
+                             dhist, dp<Counters>(s->views), dsticky));
     return GS_OK;
   };
   for (int attempt = 0;; ++attempt) {
@@ -2054,7 +2056,7 @@ gs_status refine_on_device(gs_scene* s, int nv, const gs_camera* cams, gs_pose* 
       status = fail(GS_ERR_CUDA, "refinement state upload failed");
       break;
     }
-    status = launch_update(st);
+    status = launch_update(st, false);
     if (status != GS_OK) break;
     if (iters > 1 && !s->timing) {
       // one iteration as a graph (kernel timing needs the eager path's events)
@@ -2069,7 +2071,7 @@ gs_status refine_on_device(gs_scene* s, int nv, const gs_camera* cams, gs_pose* 
       }
       gs_status est = enqueue(s, hv, ranges, n_tiles, &g, cap, nullptr, nullptr, nullptr, nullptr, true, nullptr,
                               true);
-      if (est == GS_OK) est = launch_update(cap);
+      if (est == GS_OK) est = launch_update(cap, true);
       const cudaError_t ce = cudaStreamEndCapture(cap, &graph);
       if (est == GS_OK && ce != cudaSuccess)
         est = fail(GS_ERR_CUDA, std::string("cudaStreamEndCapture: ") + cudaGetErrorString(ce));
@@ -2086,7 +2088,7 @@ gs_status refine_on_device(gs_scene* s, int nv, const gs_camera* cams, gs_pose* 
     } else {
       for (int it = 1; it < iters && status == GS_OK; ++it) {
         status = enqueue(s, hv, ranges, n_tiles, &g, st, nullptr, nullptr, nullptr, nullptr, false, nullptr, true);
-        if (status == GS_OK) status = launch_update(st);
+        if (status == GS_OK) status = launch_update(st, true);
       }
     }
     if (status != GS_OK) break;

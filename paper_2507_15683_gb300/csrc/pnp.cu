@@ -977,7 +977,8 @@ gs_status gs_pnp_solve(gs_pnp* s, const gs_camera* cam, const gs_pose* T_render,
     k_pnp_flags<<<nb, kThreads, 0, st>>>(matches, n_matches, alpha, c.W * c.H, opts->min_alpha, s->blk, s->vwords, s->st);
     PNP_CUDA(cudaGetLastError());
   }
-  PNP_CUDA(gsr::launch_dependent(!s->timing, k_pnp_scan, 1, 1024, st, s->blk, nb, s->st));
+  // (without a match there is no kernel in front that it could start behind)
+  PNP_CUDA(gsr::launch_dependent(!s->timing && nb > 0, k_pnp_scan, 1, 1024, st, s->blk, nb, s->st));
   // P3P needs the compaction's counts and bits only and runs beside the lifting
   // (phase timing keeps them in order)
   const bool fork = n_hypotheses > 0 && !s->timing;

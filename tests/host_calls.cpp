@@ -4,6 +4,7 @@
 
 #include "gsr.h"
 #include "gsr_pmm.h"
+#include "gsr_pnp.h"
 
 static int failed = 0;
 #define CHECK(x)                                                \
@@ -81,9 +82,46 @@ static void two_devices() {
   }
 }
 
+// A kernel that may start early stands directly behind another kernel of its
+// stream: also without Gaussians, without matches, and at a refinement's start.
+static void early_starts() {
+  static float image[4 * 64 * 64];
+  static int32_t matches[3 * 64];
+  static uint32_t words[3 * 8];
+  const gs_camera c = camera(64, 64);
+  for (int n : {0, 100}) {
+    gs_scene* s = scene(n);
+    const gs_outputs o{};
+    double loss, grad[6];
+    for (int timed = 0; timed < 2; ++timed) {
+      CHECK(gs_scene_set_timing(s, timed) == GS_OK);
+      for (int k = 0; k < 40; ++k) {
+        const gs_pose p = pose(k);
+        CHECK(gs_render(s, &c, &p, &o, nullptr) == GS_OK);
+        CHECK(gs_render_pose_grad(s, &c, &p, image, image, nullptr, 1.0f, nullptr, &loss, grad, nullptr) == GS_OK);
+        CHECK(gs_render_batch(s, 1, &c, &p, &o, GS_BATCH_GRAPH, nullptr) == GS_OK);
+      }
+      gs_refine_opts ro = gs_refine_defaults();
+      ro.iterations = 3;
+      gs_pose p = pose(0);
+      CHECK(gs_refine_pose(s, &c, &p, image, image, nullptr, &ro, nullptr, nullptr) == GS_OK);
+    }
+    gs_destroy_scene(s);
+  }
+  gs_pnp* q = nullptr;
+  CHECK(gs_pnp_create(64, 8, &q) == GS_OK);
+  const gs_pnp_opts po = gs_pnp_defaults();
+  const gs_pose p = pose(0);
+  gs_pnp_result r{};
+  for (int n : {0, 64})
+    for (int h : {0, 8}) CHECK(gs_pnp_solve(q, &c, &p, image, image, matches, n, words, h, &po, &r, nullptr) == GS_OK);
+  gs_pnp_destroy(q);
+}
+
 int main(int argc, char** argv) {
   const std::map<std::string, void (*)()> all = {{"batches_of_changing_size", batches_of_changing_size},
-                                                    {"two_devices", two_devices}};
+                                                    {"two_devices", two_devices},
+                                                    {"early_starts", early_starts}};
   const auto it = all.find(argc > 1 ? argv[1] : "");
   if (it == all.end()) return 2;
   it->second();
