@@ -121,14 +121,16 @@ struct VisOut {
 struct GraphCache {
   bool valid = false;
   cudaGraphExec_t exec = nullptr;
-  std::vector<char> key;       // of the capture
-  std::vector<char> last_key;  // of the last synchronous call
+  std::vector<char> key;       // of the capture; of a synchronous call, from its first plain call on
   char* host_table = nullptr;  // pinned call table (ranges + views), read by the graph's upload node
+  size_t host_bytes = 0;
   cudaEvent_t done = nullptr;
-  cudaStream_t capture = nullptr;
-  int n_views = 0;
-  uint64_t gen = 0;  // g_alloc_gen at capture
+  uint64_t gen = 0;   // g_alloc_gen at capture
+  int plain = 0;      // synchronous calls: those of this key that ran without a graph since the last capture
+  uint64_t used = 0;  // synchronous calls: number of the last one
 };
+constexpr int kSyncGraphs = 8;     // graphs of synchronous calls per scene
+constexpr int kPlainCalls = 8;     // plain calls of a key before it is captured
 
 }  // namespace
 
@@ -216,8 +218,9 @@ struct gs_scene {
   uint32_t last_tiles = 0;
   GraphCache graph;       // forward batches
   GraphCache graph_grad;  // pose-gradient batches
-  GraphCache graph_sync;  // synchronous single-view pose gradients
-  GraphCache graph_fwd;   // synchronous single-view renders
+  GraphCache graph_sync[kSyncGraphs];  // synchronous single-view renders and pose gradients, by key
+  uint64_t sync_calls = 0;
+  cudaStream_t capture_st = nullptr;
 };
 
 namespace {
@@ -803,13 +806,17 @@ gs_status check_grad_args(const float* target_rgb, const float* target_depth, fl
 
 namespace {
 
-// Replay the cached graph if the batch layout (key) is unchanged, else capture
-// a new one. Everything the capture needs is allocated before capturing.
+bool graph_ready(const GraphCache& G, const std::vector<char>& key) {
+  return G.valid && G.key == key && G.gen == g_alloc_gen.load();
+}
+
+// Replay the cached graph if the call's key is unchanged, else capture a new
+// one. Everything the capture needs is allocated before capturing.
 gs_status run_graph(gs_scene* s, GraphCache& G, const std::vector<char>& key, const std::vector<View>& hv,
                     uint64_t n_tiles, const GradIn* g, cudaStream_t st, bool copy_back = false) {
   const int n_views = (int)hv.size();
   std::vector<int4> ranges;
-  const bool ready = G.valid && G.key == key && G.gen == g_alloc_gen.load();
+  const bool ready = graph_ready(G, key);
   // the last replay has read the table, which is overwritten below, or freed for a new capture's
   if (G.exec) GS_CUDA(cudaEventSynchronize(G.done));
   GS_TRY(prepare_call(s, hv, st, ranges));  // uploads partitions on st before the graph runs
@@ -817,32 +824,37 @@ gs_status run_graph(gs_scene* s, GraphCache& G, const std::vector<char>& key, co
     if (G.exec) cudaGraphExecDestroy(G.exec);
     G.exec = nullptr;
     G.valid = false;
-    if (G.host_table) cudaFreeHost(G.host_table);
-    G.host_table = nullptr;
+    const size_t tb = table_bytes(s, n_views);
+    if (G.host_bytes < tb) {
+      if (G.host_table) cudaFreeHost(G.host_table);
+      G.host_table = nullptr;
+      G.host_bytes = 0;
+      GS_CUDA(cudaMallocHost(&G.host_table, tb));
+      G.host_bytes = tb;
+    }
     if (!G.done) GS_CUDA(cudaEventCreateWithFlags(&G.done, cudaEventDisableTiming));
-    GS_CUDA(cudaMallocHost(&G.host_table, table_bytes(s, n_views)));
-    fill_table(s, hv, ranges, G.host_table);
     GS_TRY(grow_tiles(s, n_tiles));
-    GS_TRY(ensure(s->views, table_bytes(s, n_views)));
+    GS_TRY(ensure(s->views, tb));
     if (g && !g->result) GS_TRY(ensure(s->result, (size_t)n_views * kResultStride * sizeof(double)));
     const uint64_t guess = std::max<uint64_t>(1u << 16, (uint64_t)s->n * n_views / 4);
     GS_TRY(grow_records(s, s->rec_cap ? s->rec_cap : guess, g != nullptr));
     GS_TRY(grow_pairs(s, s->pair_cap ? s->pair_cap : guess * 8));
     // capture on a private stream (the legacy default stream cannot be captured);
     // the graph is then launched on the caller's stream
-    if (!G.capture) GS_CUDA(cudaStreamCreateWithFlags(&G.capture, cudaStreamNonBlocking));
+    if (!s->capture_st) GS_CUDA(cudaStreamCreateWithFlags(&s->capture_st, cudaStreamNonBlocking));
+    const cudaStream_t cap = s->capture_st;
     GS_TRY(zero_counts(s, st));
     GS_CUDA(cudaStreamSynchronize(st));
     cudaGraph_t graph = nullptr;
-    GS_CUDA(cudaStreamBeginCapture(G.capture, cudaStreamCaptureModeThreadLocal));
-    gs_status est = enqueue(s, hv, ranges, n_tiles, g, G.capture, G.host_table, nullptr, nullptr, nullptr, true);
+    GS_CUDA(cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal));
+    gs_status est = enqueue(s, hv, ranges, n_tiles, g, cap, G.host_table, nullptr, nullptr, nullptr, true);
     if (est == GS_OK && copy_back) {  // the counters and the (loss, gradient) to the pinned host copies
-      if (cudaMemcpyAsync(s->ctr_host, s->views.p, sizeof(Counters), cudaMemcpyDeviceToHost, G.capture) != cudaSuccess ||
-          (g && cudaMemcpyAsync(s->result_host, s->result.p, 7 * sizeof(double), cudaMemcpyDeviceToHost, G.capture) !=
+      if (cudaMemcpyAsync(s->ctr_host, s->views.p, sizeof(Counters), cudaMemcpyDeviceToHost, cap) != cudaSuccess ||
+          (g && cudaMemcpyAsync(s->result_host, s->result.p, 7 * sizeof(double), cudaMemcpyDeviceToHost, cap) !=
                     cudaSuccess))
         est = fail(GS_ERR_CUDA, "cudaMemcpyAsync in the captured call failed");
     }
-    const cudaError_t ce = cudaStreamEndCapture(G.capture, &graph);
+    const cudaError_t ce = cudaStreamEndCapture(cap, &graph);
     if (est != GS_OK) {
       if (graph) cudaGraphDestroy(graph);
       return est;
@@ -852,14 +864,12 @@ gs_status run_graph(gs_scene* s, GraphCache& G, const std::vector<char>& key, co
     cudaGraphDestroy(graph);
     if (ie != cudaSuccess) return fail(GS_ERR_CUDA, std::string("cudaGraphInstantiate: ") + cudaGetErrorString(ie));
     G.key = key;
-    G.n_views = n_views;
     G.gen = g_alloc_gen.load();
     G.valid = true;
-  } else {
-    fill_table(s, hv, ranges, G.host_table);
-    s->last_views = hv;
-    s->last_tiles = (uint32_t)n_tiles;
   }
+  fill_table(s, hv, ranges, G.host_table);
+  s->last_views = hv;
+  s->last_tiles = (uint32_t)n_tiles;
   GS_TRY(zero_counts(s, st));
   GS_CUDA(cudaGraphLaunch(G.exec, st));
   GS_CUDA(cudaEventRecord(G.done, st));
@@ -873,7 +883,8 @@ void append_bytes(std::vector<char>& key, const T* p, size_t n) {
 }
 
 // What a captured call depends on besides the workspace (its generation): the
-// views' sizes, whether features are rendered, and where the results go.
+// views' sizes, whether features are rendered, whether gradients are, and where
+// the results go.
 std::vector<char> graph_key(const std::vector<View>& hv, const GradIn* g) {
   std::vector<char> key;
   char feats = 0;
@@ -883,32 +894,59 @@ std::vector<char> graph_key(const std::vector<View>& hv, const GradIn* g) {
     if (V.feats) feats = 1;
   }
   append_bytes(key, &feats, 1);
+  const char grad = g != nullptr;
+  append_bytes(key, &grad, 1);
   if (g) append_bytes(key, &g->result, 1);
   return key;
 }
 
 // A synchronous single-view call replayed from a CUDA graph: one launch instead
-// of the call's memsets, table upload, six to seven kernel launches, events and
-// read-backs. The second call in a row of the same key captures it (one whose
-// sizes change from call to call never pays for a capture). A call that
-// overflows the workspace is redone by the regrow path and the next call
-// captures again. With kernel timing on, the ordinary path runs (graphs carry
-// no timing events). A 128 x 128 render of 1,000 Gaussians: 93 -> 73 us a call.
+// of the call's table upload, six to seven kernel launches, events and
+// read-backs. A capture costs about as much as eight replays save (a 128 x 128
+// render of 1,000 Gaussians: plain 56 us, the call that captures 125, replayed
+// 47; its gradient 105, 165 and 75), so a key is captured at its ninth call: a
+// scene that is rendered a few times, or in sizes that hardly come back, pays
+// nothing, and one whose sizes return waits for the capture once in nine calls
+// at the most. kSyncGraphs keys are kept, the one not used for longest gives
+// way. A call that overflows the workspace is redone by the regrow path, and its
+// key counts plain calls again; so does one whose workspace or launch
+// configuration changed. With kernel timing on, the ordinary path runs (graphs
+// carry no timing events).
 gs_status run_sync_graphed(gs_scene* s, const std::vector<View>& hv, uint64_t n_tiles, const GradIn* g,
                            cudaStream_t st) {
   if (s->timing || hv.size() != 1 || (g && g->result)) return run_sync(s, hv, n_tiles, g, st);
-  GraphCache& G = g ? s->graph_sync : s->graph_fwd;
   std::vector<char> key = graph_key(hv, g);
-  if (G.last_key != key) {
-    G.last_key = std::move(key);
-    return run_sync(s, hv, n_tiles, g, st);
+  GraphCache* G = &s->graph_sync[0];
+  for (GraphCache& c : s->graph_sync) {
+    if (c.key == key) {
+      G = &c;
+      break;
+    }
+    if (c.used < G->used) G = &c;
   }
-  GS_TRY(run_graph(s, G, key, hv, n_tiles, g, st, true));  // the graph copies the results back
+  if (G->key != key) {
+    G->key = key;
+    G->valid = false;
+    G->plain = 0;
+  }
+  G->used = ++s->sync_calls;
+  if (!graph_ready(*G, key)) {
+    if (G->valid) {  // captured on another workspace or launch configuration
+      G->valid = false;
+      G->plain = 0;
+    }
+    if (G->plain < kPlainCalls) {
+      ++G->plain;
+      return run_sync(s, hv, n_tiles, g, st);
+    }
+  }
+  GS_TRY(run_graph(s, *G, key, hv, n_tiles, g, st, true));  // the graph copies the results back
   GS_CUDA(cudaStreamSynchronize(st));
   const Counters& c = *s->ctr_host;
   if (c.error) return fail(GS_ERR_INTERNAL, "device consistency check failed: the binning handed out a pair slot past the scanned tile counts");
   if (c.overflow) {
-    G.valid = false;
+    G->valid = false;
+    G->plain = 0;
     return run_sync(s, hv, n_tiles, g, st);
   }
   return GS_OK;
@@ -1095,12 +1133,14 @@ void gs_destroy_scene(gs_scene* s) {
   if (!s) return;
   cudaSetDevice(s->device);
   cudaDeviceSynchronize();
-  for (GraphCache* G : {&s->graph, &s->graph_grad, &s->graph_sync, &s->graph_fwd}) {
+  std::vector<GraphCache*> graphs = {&s->graph, &s->graph_grad};
+  for (GraphCache& G : s->graph_sync) graphs.push_back(&G);
+  for (GraphCache* G : graphs) {
     if (G->exec) cudaGraphExecDestroy(G->exec);
     if (G->host_table) cudaFreeHost(G->host_table);
     if (G->done) cudaEventDestroy(G->done);
-    if (G->capture) cudaStreamDestroy(G->capture);
   }
+  if (s->capture_st) cudaStreamDestroy(s->capture_st);
   for (auto& tc : s->ev_pending)
     for (cudaEvent_t e : tc.ev) cudaEventDestroy(e);
   for (auto& ev : s->ev_free)

@@ -118,10 +118,41 @@ static void early_starts() {
   gs_pnp_destroy(q);
 }
 
+static void render(gs_scene* s, const gs_camera& c) {
+  const gs_outputs o{};
+  const gs_pose p = pose(0);
+  CHECK(gs_render(s, &c, &p, &o, nullptr) == GS_OK);
+}
+
+// Synchronous renders are captured once their size has come up often, and only
+// once: not again for a size that comes back, and never for sizes that are many.
+static void sizes_in_pairs() {
+  gs_scene* s = scene(100);
+  fake::count.clear();
+  for (int k = 0; k < 100; ++k)
+    for (int w : {64, 64, 96, 96}) render(s, camera(w, 64));
+  CHECK(fake::count["captures"] == 2);
+  CHECK(fake::count["replays"] >= 380);
+  const int mallocs = fake::count["cudaMallocHost"];
+  for (int k = 0; k < 400; ++k) render(s, camera(32 + 16 * (k / 2 % 20), 32));  // 20 sizes
+  CHECK(fake::count["captures"] == 2);
+  CHECK(fake::count["cudaMallocHost"] == mallocs);
+  for (int w = 0; w < 3; ++w)  // a size rendered twice by each of many scenes
+    for (int k = 0; k < 10; ++k) {
+      gs_scene* t = scene(10);
+      render(t, camera(64, 64));
+      render(t, camera(64, 64));
+      gs_destroy_scene(t);
+    }
+  CHECK(fake::count["captures"] == 2);
+  gs_destroy_scene(s);
+}
+
 int main(int argc, char** argv) {
   const std::map<std::string, void (*)()> all = {{"batches_of_changing_size", batches_of_changing_size},
                                                     {"two_devices", two_devices},
-                                                    {"early_starts", early_starts}};
+                                                    {"early_starts", early_starts},
+                                                    {"sizes_in_pairs", sizes_in_pairs}};
   const auto it = all.find(argc > 1 ? argv[1] : "");
   if (it == all.end()) return 2;
   it->second();

@@ -11,6 +11,37 @@ pytestmark = pytest.mark.gpu
 CALLS = 40  # more plain calls than any size takes before it is captured
 
 
+def _scene(n=20000):
+    return synth.aerial_scene(5, n, extent=(0.0, 200.0, 0.0, 200.0), n_clusters=20)
+
+
+def _pose(k):
+    return synth.look_pose((100.0 + 5 * k, 40.0, 60.0), 0.1 * k, 0.5)
+
+
+def test_sizes_and_kinds_in_turn(gsr):
+    # ten sizes, renders and gradients: more keys than a scene keeps graphs, so that graphs are captured, replayed,
+    # given up and captured again; every call has the bits of a scene that has captured nothing
+    cams = [synth.camera(w, h, 0.7 * w) for w in (16, 100, 240, 333, 960) for h in (16, 251)]
+    S = gsr.Scene(_scene())
+    want, grads = [], []
+    for c in cams:
+        F = gsr.Scene(_scene())
+        want.append([F.render(c, _pose(k)) for k in range(2)])
+        grads.append(F.render_pose_grad(c, _pose(1), want[-1][0]["rgb"], want[-1][0]["depth"]))
+        F.close()
+    for runs in (2, 12, 2, 12):
+        for c, w, (loss, grad) in zip(cams, want, grads):
+            for k in range(runs):
+                out = S.render(c, _pose(k & 1))
+                for name, v in w[k & 1].items():
+                    assert torch.equal(out[name], v), (c, k, name)
+                got = S.render_pose_grad(c, _pose(1), w[0]["rgb"], w[0]["depth"])
+                assert got[0] == loss
+                np.testing.assert_array_equal(got[1], grad)
+    S.close()
+
+
 def test_empty_scene(gsr):
     S = gsr.Scene(synth.tiny_scene(0, n=0))
     cam = synth.camera(48, 33, 40.0)
