@@ -8,7 +8,6 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
-#include <atomic>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -47,30 +46,6 @@ struct DevBuf {
   void* p = nullptr;
   size_t bytes = 0;
 };
-
-// Bumped by every device (re)allocation of a workspace buffer and by every
-// change of a launch configuration: a captured graph holds the buffers'
-// addresses and the launch shapes, and is replayed only while this is
-// unchanged since its capture.
-std::atomic<uint64_t> g_alloc_gen{0};
-
-gs_status ensure(DevBuf& b, size_t bytes) {
-  if (b.bytes >= bytes && b.p) return GS_OK;
-  g_alloc_gen.fetch_add(1);
-  if (b.p) cudaFree(b.p);
-  b.p = nullptr;
-  b.bytes = 0;
-  const size_t alloc = std::max<size_t>(bytes, 256);
-  const cudaError_t e = cudaMalloc(&b.p, alloc);
-  if (e != cudaSuccess) {
-    cudaGetLastError();
-    b.p = nullptr;
-    return fail(e == cudaErrorMemoryAllocation ? GS_ERR_OOM : GS_ERR_CUDA,
-                std::string("cudaMalloc(") + std::to_string(alloc) + "): " + cudaGetErrorString(e));
-  }
-  b.bytes = alloc;
-  return GS_OK;
-}
 
 void release(DevBuf& b) {
   if (b.p) cudaFree(b.p);
@@ -125,7 +100,7 @@ struct GraphCache {
   char* host_table = nullptr;  // pinned call table (ranges + views), read by the graph's upload node
   size_t host_bytes = 0;
   cudaEvent_t done = nullptr;
-  uint64_t gen = 0;   // g_alloc_gen at capture
+  uint64_t gen = 0;   // the scene's alloc_gen at capture
   int plain = 0;      // synchronous calls: those of this key that ran without a graph since the last capture
   uint64_t used = 0;  // synchronous calls: number of the last one
 };
@@ -169,6 +144,11 @@ struct gs_scene {
   uint4* h_feat = nullptr;
   int64_t h2d_bytes = 0;
   int last_active = 0;
+  // Bumped by every device (re)allocation of a workspace buffer and by every
+  // change of a launch configuration: a captured graph holds the buffers'
+  // addresses and the launch shapes, and is replayed only while this is
+  // unchanged since its capture.
+  uint64_t alloc_gen = 0;
   // workspace
   DevBuf rec_a, rec_b, rec_c, rec_m, rec_j;
   uint32_t rec_cap = 0, jac_cap = 0;
@@ -224,6 +204,24 @@ struct gs_scene {
 };
 
 namespace {
+
+gs_status ensure(gs_scene* s, DevBuf& b, size_t bytes) {
+  if (b.bytes >= bytes && b.p) return GS_OK;
+  ++s->alloc_gen;
+  if (b.p) cudaFree(b.p);
+  b.p = nullptr;
+  b.bytes = 0;
+  const size_t alloc = std::max<size_t>(bytes, 256);
+  const cudaError_t e = cudaMalloc(&b.p, alloc);
+  if (e != cudaSuccess) {
+    cudaGetLastError();
+    b.p = nullptr;
+    return fail(e == cudaErrorMemoryAllocation ? GS_ERR_OOM : GS_ERR_CUDA,
+                std::string("cudaMalloc(") + std::to_string(alloc) + "): " + cudaGetErrorString(e));
+  }
+  b.bytes = alloc;
+  return GS_OK;
+}
 
 // Call-shape key of a launch configuration: the views' sizes as a sorted
 // multiset, "WxH*count" joined by commas.
@@ -295,14 +293,14 @@ gs_status grow_records(gs_scene* s, uint64_t rec_cap, bool grad) {
   rec_cap = std::min<uint64_t>(rec_cap, 0x7fffffffull);
   rec_cap = (rec_cap + kRecRegions - 1) / kRecRegions * kRecRegions;  // equal segments
   if (rec_cap > s->rec_cap) {
-    GS_TRY(ensure(s->rec_a, rec_cap * sizeof(float4)));
-    GS_TRY(ensure(s->rec_b, rec_cap * sizeof(float4)));
-    GS_TRY(ensure(s->rec_c, rec_cap * sizeof(float4)));
-    GS_TRY(ensure(s->rec_m, rec_cap * sizeof(uint4)));
+    GS_TRY(ensure(s, s->rec_a, rec_cap * sizeof(float4)));
+    GS_TRY(ensure(s, s->rec_b, rec_cap * sizeof(float4)));
+    GS_TRY(ensure(s, s->rec_c, rec_cap * sizeof(float4)));
+    GS_TRY(ensure(s, s->rec_m, rec_cap * sizeof(uint4)));
     s->rec_cap = (uint32_t)rec_cap;
   }
   if (grad && s->jac_cap < s->rec_cap) {
-    GS_TRY(ensure(s->rec_j, (size_t)s->rec_cap * kJacStride * sizeof(float)));
+    GS_TRY(ensure(s, s->rec_j, (size_t)s->rec_cap * kJacStride * sizeof(float)));
     s->jac_cap = s->rec_cap;
   }
   return GS_OK;
@@ -311,8 +309,8 @@ gs_status grow_records(gs_scene* s, uint64_t rec_cap, bool grad) {
 gs_status grow_pairs(gs_scene* s, uint64_t pair_cap) {
   pair_cap = std::min<uint64_t>(pair_cap, 0xffffffffull);
   if (pair_cap > s->pair_cap) {
-    GS_TRY(ensure(s->pairs, pair_cap * sizeof(uint2)));
-    GS_TRY(ensure(s->pairs_tmp, pair_cap * sizeof(uint2)));
+    GS_TRY(ensure(s, s->pairs, pair_cap * sizeof(uint2)));
+    GS_TRY(ensure(s, s->pairs_tmp, pair_cap * sizeof(uint2)));
     s->pair_cap = (uint32_t)pair_cap;
   }
   return GS_OK;
@@ -322,10 +320,10 @@ gs_status grow_tiles(gs_scene* s, uint64_t n_tiles) {
   if (n_tiles + 1 > s->tile_cap) {
     const uint64_t cap = n_tiles + 1;
     s->counts_zero = false;
-    GS_TRY(ensure(s->tile_ctr, ctr_words(cap) * sizeof(uint32_t)));
-    GS_TRY(ensure(s->tile_offset, cap * sizeof(uint32_t)));
-    GS_TRY(ensure(s->partials, cap * kPartialStride * sizeof(double)));
-    GS_TRY(ensure(s->chunks, cap * (kPartialStride * sizeof(double) + sizeof(uint32_t))));
+    GS_TRY(ensure(s, s->tile_ctr, ctr_words(cap) * sizeof(uint32_t)));
+    GS_TRY(ensure(s, s->tile_offset, cap * sizeof(uint32_t)));
+    GS_TRY(ensure(s, s->partials, cap * kPartialStride * sizeof(double)));
+    GS_TRY(ensure(s, s->chunks, cap * (kPartialStride * sizeof(double) + sizeof(uint32_t))));
     s->tile_cap = (uint32_t)cap;
   }
   return GS_OK;
@@ -444,8 +442,8 @@ gs_status enqueue(gs_scene* s, const std::vector<View>& hv, const std::vector<in
   const int nv = (int)hv.size();
   const bool jac = g != nullptr || vis != nullptr;  // per-record pose Jacobian
   GS_TRY(grow_tiles(s, n_tiles));
-  GS_TRY(ensure(s->views, table_bytes(s, nv)));
-  if (g && !g->result) GS_TRY(ensure(s->result, (size_t)nv * kResultStride * sizeof(double)));
+  GS_TRY(ensure(s, s->views, table_bytes(s, nv)));
+  if (g && !g->result) GS_TRY(ensure(s, s->result, (size_t)nv * kResultStride * sizeof(double)));
   if (s->rec_cap == 0) {
     const uint64_t guess = std::max<uint64_t>(1u << 16, (uint64_t)s->n * nv / 4);
     GS_TRY(grow_records(s, guess, jac));
@@ -455,8 +453,8 @@ gs_status enqueue(gs_scene* s, const std::vector<View>& hv, const std::vector<in
   }
   if (s->pair_cap == 0) GS_TRY(grow_pairs(s, (uint64_t)s->rec_cap * 8));
   if (vis) {
-    GS_TRY(ensure(s->vis_acc, (size_t)s->rec_cap * kVisAcc * sizeof(float)));
-    GS_TRY(ensure(s->vis_blk, ((size_t)s->n / kVisBlock + 1) * sizeof(uint32_t)));
+    GS_TRY(ensure(s, s->vis_acc, (size_t)s->rec_cap * kVisAcc * sizeof(float)));
+    GS_TRY(ensure(s, s->vis_blk, ((size_t)s->n / kVisBlock + 1) * sizeof(uint32_t)));
   }
   View* dviews = reinterpret_cast<View*>(static_cast<char*>(s->views.p) + table_views_off(s));
   if (keep_table) {
@@ -806,8 +804,8 @@ gs_status check_grad_args(const float* target_rgb, const float* target_depth, fl
 
 namespace {
 
-bool graph_ready(const GraphCache& G, const std::vector<char>& key) {
-  return G.valid && G.key == key && G.gen == g_alloc_gen.load();
+bool graph_ready(const gs_scene* s, const GraphCache& G, const std::vector<char>& key) {
+  return G.valid && G.key == key && G.gen == s->alloc_gen;
 }
 
 // Replay the cached graph if the call's key is unchanged, else capture a new
@@ -816,7 +814,7 @@ gs_status run_graph(gs_scene* s, GraphCache& G, const std::vector<char>& key, co
                     uint64_t n_tiles, const GradIn* g, cudaStream_t st, bool copy_back = false) {
   const int n_views = (int)hv.size();
   std::vector<int4> ranges;
-  const bool ready = graph_ready(G, key);
+  const bool ready = graph_ready(s, G, key);
   // the last replay has read the table, which is overwritten below, or freed for a new capture's
   if (G.exec) GS_CUDA(cudaEventSynchronize(G.done));
   GS_TRY(prepare_call(s, hv, st, ranges));  // uploads partitions on st before the graph runs
@@ -834,8 +832,8 @@ gs_status run_graph(gs_scene* s, GraphCache& G, const std::vector<char>& key, co
     }
     if (!G.done) GS_CUDA(cudaEventCreateWithFlags(&G.done, cudaEventDisableTiming));
     GS_TRY(grow_tiles(s, n_tiles));
-    GS_TRY(ensure(s->views, tb));
-    if (g && !g->result) GS_TRY(ensure(s->result, (size_t)n_views * kResultStride * sizeof(double)));
+    GS_TRY(ensure(s, s->views, tb));
+    if (g && !g->result) GS_TRY(ensure(s, s->result, (size_t)n_views * kResultStride * sizeof(double)));
     const uint64_t guess = std::max<uint64_t>(1u << 16, (uint64_t)s->n * n_views / 4);
     GS_TRY(grow_records(s, s->rec_cap ? s->rec_cap : guess, g != nullptr));
     GS_TRY(grow_pairs(s, s->pair_cap ? s->pair_cap : guess * 8));
@@ -864,7 +862,7 @@ gs_status run_graph(gs_scene* s, GraphCache& G, const std::vector<char>& key, co
     cudaGraphDestroy(graph);
     if (ie != cudaSuccess) return fail(GS_ERR_CUDA, std::string("cudaGraphInstantiate: ") + cudaGetErrorString(ie));
     G.key = key;
-    G.gen = g_alloc_gen.load();
+    G.gen = s->alloc_gen;
     G.valid = true;
   }
   fill_table(s, hv, ranges, G.host_table);
@@ -930,7 +928,7 @@ gs_status run_sync_graphed(gs_scene* s, const std::vector<View>& hv, uint64_t n_
     G->plain = 0;
   }
   G->used = ++s->sync_calls;
-  if (!graph_ready(*G, key)) {
+  if (!graph_ready(s, *G, key)) {
     if (G->valid) {  // captured on another workspace or launch configuration
       G->valid = false;
       G->plain = 0;
@@ -1005,11 +1003,11 @@ gs_status gs_create_scene(const gs_scene_desc* d, gs_scene** out) {
   if (e != cudaSuccess) return cleanup(fail(GS_ERR_CUDA, std::string("stream / event creation: ") + cudaGetErrorString(e)));
   const size_t n = (size_t)d->n;
   gs_status st;
-  if ((st = ensure(s->pos, n * sizeof(float4))) != GS_OK) return cleanup(st);
-  if ((st = ensure(s->cov, 2 * n * sizeof(float4))) != GS_OK) return cleanup(st);
-  if ((st = ensure(s->sh, n * s->nsh4 * sizeof(float4))) != GS_OK) return cleanup(st);
-  if (s->feat_dim && (st = ensure(s->feat, n * 4 * sizeof(uint4))) != GS_OK) return cleanup(st);
-  if ((st = ensure(s->result, 8 * sizeof(double))) != GS_OK) return cleanup(st);
+  if ((st = ensure(s, s->pos, n * sizeof(float4))) != GS_OK) return cleanup(st);
+  if ((st = ensure(s, s->cov, 2 * n * sizeof(float4))) != GS_OK) return cleanup(st);
+  if ((st = ensure(s, s->sh, n * s->nsh4 * sizeof(float4))) != GS_OK) return cleanup(st);
+  if (s->feat_dim && (st = ensure(s, s->feat, n * 4 * sizeof(uint4))) != GS_OK) return cleanup(st);
+  if ((st = ensure(s, s->result, 8 * sizeof(double))) != GS_OK) return cleanup(st);
   if (cudaMallocHost(&s->ctr_host, sizeof(Counters)) != cudaSuccess ||
       cudaMallocHost(&s->result_host, 8 * sizeof(double)) != cudaSuccess) {
     cudaGetLastError();
@@ -1057,7 +1055,7 @@ gs_status gs_create_scene(const gs_scene_desc* d, gs_scene** out) {
       s->parts.push_back(P);
     }
   }
-  if ((st = ensure(s->views, table_bytes(s, 1))) != GS_OK) return cleanup(st);
+  if ((st = ensure(s, s->views, table_bytes(s, 1))) != GS_OK) return cleanup(st);
   if ((e = cudaMemset(s->views.p, 0, kCtrBytes)) != cudaSuccess)
     return cleanup(fail(GS_ERR_CUDA, std::string("cudaMemset: ") + cudaGetErrorString(e)));
   s->streaming = !d->device_resident && d->n_partitions > 0 && n > 0;
@@ -1093,7 +1091,7 @@ gs_status gs_create_scene(const gs_scene_desc* d, gs_scene** out) {
     if (!d->device_resident) {
       const size_t fb = s->feat_dim ? n * 32 * sizeof(uint16_t) : 0;
       const size_t bytes = n * (3 + 3 + 4 + 1 + K3) * sizeof(float) + fb;
-      if ((st = ensure(staging, bytes)) != GS_OK) return cleanup(st);
+      if ((st = ensure(s, staging, bytes)) != GS_OK) return cleanup(st);
       char* p = static_cast<char*>(staging.p);
       auto put = [&](const void* src, size_t b) {
         void* dst = p;
@@ -1274,7 +1272,7 @@ gs_status gs_render_pose_grad_host(gs_scene* s, const gs_camera* cam, const gs_p
     }
   }
   // pageable targets: uploaded by the copy engine, in bands
-  GS_TRY(ensure(s->targets, (pixel_weight ? 5 : 4) * P * sizeof(float)));
+  GS_TRY(ensure(s, s->targets, (pixel_weight ? 5 : 4) * P * sizeof(float)));
   if (!s->copy_st) GS_CUDA(cudaStreamCreateWithFlags(&s->copy_st, cudaStreamNonBlocking));
   if (!s->ev_call) GS_CUDA(cudaEventCreateWithFlags(&s->ev_call, cudaEventDisableTiming));
   if (!s->ev_targets) GS_CUDA(cudaEventCreateWithFlags(&s->ev_targets, cudaEventDisableTiming));
@@ -1493,9 +1491,9 @@ gs_status gs_visibility(gs_scene* s, const gs_camera* cam, const gs_pose* pose, 
   GS_TRY(check_cam(*cam));
   const cudaStream_t st = (cudaStream_t)stream;
   const size_t P = (size_t)cam->width * cam->height;
-  GS_TRY(ensure(s->vis_T, P * sizeof(float)));
-  GS_TRY(ensure(s->vis_last, P * sizeof(uint32_t)));
-  if (!uv) GS_TRY(ensure(s->vis_uv, (size_t)std::max<int64_t>(s->n, 1) * sizeof(float2)));
+  GS_TRY(ensure(s, s->vis_T, P * sizeof(float)));
+  GS_TRY(ensure(s, s->vis_last, P * sizeof(uint32_t)));
+  if (!uv) GS_TRY(ensure(s, s->vis_uv, (size_t)std::max<int64_t>(s->n, 1) * sizeof(float2)));
   // the in-image test covers every Gaussian: a streamed scene becomes resident
   for (Part& Pt : s->parts) GS_TRY(make_resident(s, Pt, st));
   gs_outputs o{};
@@ -1570,7 +1568,7 @@ gs_status set_cfg(gs_scene* s, int mode, const std::string& key, int variant, in
   c.variant[mode] = variant;
   c.per_sm[mode] = per_sm;
   c.grid_mult[mode] = grid_mult;
-  g_alloc_gen.fetch_add(1);  // captured graphs hold the old launch shapes
+  ++s->alloc_gen;  // captured graphs hold the old launch shapes
   return GS_OK;
 }
 
@@ -1620,7 +1618,7 @@ gs_status gs_autotune(gs_scene* s, int mode, int n_views, const gs_camera* cams,
   for (int v = 0; v < n_views; ++v) {
     const size_t P = (size_t)cams[v].width * cams[v].height;
     const size_t nf = mode == kModeFwdFeat ? 32 : 0;
-    const gs_status e = ensure(bufs[v], (6 + nf) * P * sizeof(float));
+    const gs_status e = ensure(s, bufs[v], (6 + nf) * P * sizeof(float));
     if (e != GS_OK) {
       free_all();
       return e;
@@ -1723,11 +1721,11 @@ gs_status gs_autotune(gs_scene* s, int mode, int n_views, const gs_camera* cams,
   free_all();
   if (err != GS_OK) {
     s->launch[key] = saved;
-    g_alloc_gen.fetch_add(1);
+    ++s->alloc_gen;
     return err;
   }
   s->launch[key] = best;
-  g_alloc_gen.fetch_add(1);  // captured graphs hold the old launch shapes
+  ++s->alloc_gen;  // captured graphs hold the old launch shapes
   if (result) {
     fill_launch(best, mode, &result->best);
     result->ms_default = ms_default;

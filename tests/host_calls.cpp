@@ -148,11 +148,42 @@ static void sizes_in_pairs() {
   gs_destroy_scene(s);
 }
 
+// A scene's graphs outlive whatever other scenes allocate or are told to launch.
+static void other_scenes() {
+  gs_scene* s = scene(100);
+  const gs_camera c = camera(64, 64);
+  const gs_pose p[2] = {pose(0), pose(1)};
+  const gs_outputs o[2] = {};
+  const gs_camera cs[2] = {c, c};
+  CHECK(gs_render_batch(s, 2, cs, p, o, GS_BATCH_GRAPH, nullptr) == GS_OK);
+  for (int k = 0; k < 40; ++k) render(s, c);
+  fake::count.clear();
+  for (int k = 0; k < 40; ++k) {
+    gs_scene* t = scene(10);
+    render(t, camera(64 + 16 * k, 64));
+    gs_launch cfg{};
+    cfg.grid_mult = 4;
+    CHECK(gs_scene_set_launch(t, GS_MODE_FORWARD, 1, &c, &cfg) == GS_OK);
+    gs_destroy_scene(t);
+    render(s, c);
+    CHECK(gs_render_batch(s, 2, cs, p, o, GS_BATCH_GRAPH, nullptr) == GS_OK);
+  }
+  CHECK(fake::count["captures"] == 0);
+  CHECK(fake::count["replays"] == 80);
+  gs_launch cfg{};
+  cfg.grid_mult = 4;
+  CHECK(gs_scene_set_launch(s, GS_MODE_FORWARD, 1, &c, &cfg) == GS_OK);  // its own: captured again
+  for (int k = 0; k < 40; ++k) render(s, c);
+  CHECK(fake::count["captures"] == 1);
+  gs_destroy_scene(s);
+}
+
 int main(int argc, char** argv) {
   const std::map<std::string, void (*)()> all = {{"batches_of_changing_size", batches_of_changing_size},
                                                     {"two_devices", two_devices},
                                                     {"early_starts", early_starts},
-                                                    {"sizes_in_pairs", sizes_in_pairs}};
+                                                    {"sizes_in_pairs", sizes_in_pairs},
+                                                    {"other_scenes", other_scenes}};
   const auto it = all.find(argc > 1 ? argv[1] : "");
   if (it == all.end()) return 2;
   it->second();
