@@ -808,62 +808,77 @@ bool graph_ready(const gs_scene* s, const GraphCache& G, const std::vector<char>
   return G.valid && G.key == key && G.gen == s->alloc_gen;
 }
 
-// Replay the cached graph if the call's key is unchanged, else capture a new
-// one. Everything the capture needs is allocated before capturing.
-gs_status run_graph(gs_scene* s, GraphCache& G, const std::vector<char>& key, const std::vector<View>& hv,
-                    uint64_t n_tiles, const GradIn* g, cudaStream_t st, bool copy_back = false) {
+// Capture the call into G, whose last replay (if any) has ended. Everything the
+// capture needs is allocated before capturing.
+gs_status capture_graph(gs_scene* s, GraphCache& G, const std::vector<char>& key, const std::vector<View>& hv,
+                        const std::vector<int4>& ranges, uint64_t n_tiles, const GradIn* g, cudaStream_t st,
+                        bool copy_back) {
   const int n_views = (int)hv.size();
+  if (G.exec) cudaGraphExecDestroy(G.exec);
+  G.exec = nullptr;
+  G.valid = false;
+  const size_t tb = table_bytes(s, n_views);
+  if (G.host_bytes < tb) {
+    if (G.host_table) cudaFreeHost(G.host_table);
+    G.host_table = nullptr;
+    G.host_bytes = 0;
+    GS_CUDA(cudaMallocHost(&G.host_table, tb));
+    G.host_bytes = tb;
+  }
+  if (!G.done) GS_CUDA(cudaEventCreateWithFlags(&G.done, cudaEventDisableTiming));
+  GS_TRY(grow_tiles(s, n_tiles));
+  GS_TRY(ensure(s, s->views, tb));
+  if (g && !g->result) GS_TRY(ensure(s, s->result, (size_t)n_views * kResultStride * sizeof(double)));
+  const uint64_t guess = std::max<uint64_t>(1u << 16, (uint64_t)s->n * n_views / 4);
+  GS_TRY(grow_records(s, s->rec_cap ? s->rec_cap : guess, g != nullptr));
+  GS_TRY(grow_pairs(s, s->pair_cap ? s->pair_cap : guess * 8));
+  // capture on a private stream (the legacy default stream cannot be captured);
+  // the graph is then launched on the caller's stream
+  if (!s->capture_st) GS_CUDA(cudaStreamCreateWithFlags(&s->capture_st, cudaStreamNonBlocking));
+  const cudaStream_t cap = s->capture_st;
+  GS_TRY(zero_counts(s, st));
+  GS_CUDA(cudaStreamSynchronize(st));
+  cudaGraph_t graph = nullptr;
+  GS_CUDA(cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal));
+  gs_status est = enqueue(s, hv, ranges, n_tiles, g, cap, G.host_table, nullptr, nullptr, nullptr, true);
+  if (est == GS_OK && copy_back) {  // the counters and the (loss, gradient) to the pinned host copies
+    if (cudaMemcpyAsync(s->ctr_host, s->views.p, sizeof(Counters), cudaMemcpyDeviceToHost, cap) != cudaSuccess ||
+        (g && cudaMemcpyAsync(s->result_host, s->result.p, 7 * sizeof(double), cudaMemcpyDeviceToHost, cap) !=
+                  cudaSuccess))
+      est = fail(GS_ERR_CUDA, "cudaMemcpyAsync in the captured call failed");
+  }
+  const cudaError_t ce = cudaStreamEndCapture(cap, &graph);
+  if (est != GS_OK) {
+    if (graph) cudaGraphDestroy(graph);
+    return est;
+  }
+  if (ce != cudaSuccess) return fail(GS_ERR_CUDA, std::string("cudaStreamEndCapture: ") + cudaGetErrorString(ce));
+  const cudaError_t ie = cudaGraphInstantiate(&G.exec, graph, 0);
+  cudaGraphDestroy(graph);
+  if (ie != cudaSuccess) {
+    G.exec = nullptr;
+    return fail(GS_ERR_CUDA, std::string("cudaGraphInstantiate: ") + cudaGetErrorString(ie));
+  }
+  G.key = key;
+  G.gen = s->alloc_gen;
+  G.valid = true;
+  return GS_OK;
+}
+
+// Replay the cached graph if the call's key is unchanged, else capture a new
+// one. With `captured`, a capture that fails is not an error: *captured is then
+// false and nothing was launched.
+gs_status run_graph(gs_scene* s, GraphCache& G, const std::vector<char>& key, const std::vector<View>& hv,
+                    uint64_t n_tiles, const GradIn* g, cudaStream_t st, bool copy_back = false,
+                    bool* captured = nullptr) {
   std::vector<int4> ranges;
-  const bool ready = graph_ready(s, G, key);
   // the last replay has read the table, which is overwritten below, or freed for a new capture's
   if (G.exec) GS_CUDA(cudaEventSynchronize(G.done));
   GS_TRY(prepare_call(s, hv, st, ranges));  // uploads partitions on st before the graph runs
-  if (!ready) {
-    if (G.exec) cudaGraphExecDestroy(G.exec);
-    G.exec = nullptr;
-    G.valid = false;
-    const size_t tb = table_bytes(s, n_views);
-    if (G.host_bytes < tb) {
-      if (G.host_table) cudaFreeHost(G.host_table);
-      G.host_table = nullptr;
-      G.host_bytes = 0;
-      GS_CUDA(cudaMallocHost(&G.host_table, tb));
-      G.host_bytes = tb;
-    }
-    if (!G.done) GS_CUDA(cudaEventCreateWithFlags(&G.done, cudaEventDisableTiming));
-    GS_TRY(grow_tiles(s, n_tiles));
-    GS_TRY(ensure(s, s->views, tb));
-    if (g && !g->result) GS_TRY(ensure(s, s->result, (size_t)n_views * kResultStride * sizeof(double)));
-    const uint64_t guess = std::max<uint64_t>(1u << 16, (uint64_t)s->n * n_views / 4);
-    GS_TRY(grow_records(s, s->rec_cap ? s->rec_cap : guess, g != nullptr));
-    GS_TRY(grow_pairs(s, s->pair_cap ? s->pair_cap : guess * 8));
-    // capture on a private stream (the legacy default stream cannot be captured);
-    // the graph is then launched on the caller's stream
-    if (!s->capture_st) GS_CUDA(cudaStreamCreateWithFlags(&s->capture_st, cudaStreamNonBlocking));
-    const cudaStream_t cap = s->capture_st;
-    GS_TRY(zero_counts(s, st));
-    GS_CUDA(cudaStreamSynchronize(st));
-    cudaGraph_t graph = nullptr;
-    GS_CUDA(cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal));
-    gs_status est = enqueue(s, hv, ranges, n_tiles, g, cap, G.host_table, nullptr, nullptr, nullptr, true);
-    if (est == GS_OK && copy_back) {  // the counters and the (loss, gradient) to the pinned host copies
-      if (cudaMemcpyAsync(s->ctr_host, s->views.p, sizeof(Counters), cudaMemcpyDeviceToHost, cap) != cudaSuccess ||
-          (g && cudaMemcpyAsync(s->result_host, s->result.p, 7 * sizeof(double), cudaMemcpyDeviceToHost, cap) !=
-                    cudaSuccess))
-        est = fail(GS_ERR_CUDA, "cudaMemcpyAsync in the captured call failed");
-    }
-    const cudaError_t ce = cudaStreamEndCapture(cap, &graph);
-    if (est != GS_OK) {
-      if (graph) cudaGraphDestroy(graph);
-      return est;
-    }
-    if (ce != cudaSuccess) return fail(GS_ERR_CUDA, std::string("cudaStreamEndCapture: ") + cudaGetErrorString(ce));
-    const cudaError_t ie = cudaGraphInstantiate(&G.exec, graph, 0);
-    cudaGraphDestroy(graph);
-    if (ie != cudaSuccess) return fail(GS_ERR_CUDA, std::string("cudaGraphInstantiate: ") + cudaGetErrorString(ie));
-    G.key = key;
-    G.gen = s->alloc_gen;
-    G.valid = true;
+  if (!graph_ready(s, G, key)) {
+    const gs_status cst = capture_graph(s, G, key, hv, ranges, n_tiles, g, st, copy_back);
+    if (captured) *captured = cst == GS_OK;
+    if (cst != GS_OK) return captured ? GS_OK : cst;
   }
   fill_table(s, hv, ranges, G.host_table);
   s->last_views = hv;
@@ -908,7 +923,7 @@ std::vector<char> graph_key(const std::vector<View>& hv, const GradIn* g) {
 // at the most. kSyncGraphs keys are kept, the one not used for longest gives
 // way. A call that overflows the workspace is redone by the regrow path, and its
 // key counts plain calls again; so does one whose workspace or launch
-// configuration changed. With kernel timing on, the ordinary path runs (graphs
+// configuration changed, or whose capture failed. With kernel timing on, the ordinary path runs (graphs
 // carry no timing events).
 gs_status run_sync_graphed(gs_scene* s, const std::vector<View>& hv, uint64_t n_tiles, const GradIn* g,
                            cudaStream_t st) {
@@ -938,7 +953,14 @@ gs_status run_sync_graphed(gs_scene* s, const std::vector<View>& hv, uint64_t n_
       return run_sync(s, hv, n_tiles, g, st);
     }
   }
-  GS_TRY(run_graph(s, *G, key, hv, n_tiles, g, st, true));  // the graph copies the results back
+  bool captured = true;
+  GS_TRY(run_graph(s, *G, key, hv, n_tiles, g, st, true, &captured));  // the graph copies the results back
+  if (!captured) {  // no memory for it: the call needs none of it
+    cudaGetLastError();
+    g_err.clear();
+    G->plain = 0;
+    return run_sync(s, hv, n_tiles, g, st);
+  }
   GS_CUDA(cudaStreamSynchronize(st));
   const Counters& c = *s->ctr_host;
   if (c.error) return fail(GS_ERR_INTERNAL, "device consistency check failed: the binning handed out a pair slot past the scanned tile counts");

@@ -48,14 +48,10 @@ inline std::map<int, int> occupancy = {{0, 4}, {1, 3}};
 inline Stream legacy;
 inline thread_local int device = 0;
 inline thread_local cudaError_t last_error = cudaSuccess;
-inline thread_local cudaStreamCaptureMode mode = cudaStreamCaptureModeGlobal;
-inline bool other_capture = false;  // another thread captures in global mode
+inline bool no_pinned = false, no_graphs = false;  // no memory for them
 
 inline void violate(const std::string& s) { violations.push_back(s); }
 inline Stream* of(cudaStream_t s) { return s ? reinterpret_cast<Stream*>(s) : &legacy; }
-
-// calls that a thread in global mode may not make while another thread captures in that mode
-inline bool refused() { return other_capture && mode == cudaStreamCaptureModeGlobal; }
 
 inline void execute(const Op& o) {
   if (o.kind == kSet) std::memset(o.dst, o.value, o.bytes);
@@ -191,13 +187,11 @@ cudaError_t cudaDeviceSynchronize() {
 }
 
 cudaError_t cudaMalloc(void** p, size_t n) {
-  if (fake::refused()) return cudaErrorStreamCaptureUnsupported;
   fake::count["cudaMalloc"]++;
   *p = std::calloc(1, n);
   return *p ? cudaSuccess : cudaErrorMemoryAllocation;
 }
 cudaError_t cudaFree(void* p) {  // waits for the device
-  if (fake::refused()) return cudaErrorStreamCaptureUnsupported;
   fake::drain();
   std::free(p);
   return cudaSuccess;
@@ -205,15 +199,14 @@ cudaError_t cudaFree(void* p) {  // waits for the device
 cudaError_t cudaMallocAsync(void** p, size_t n, cudaStream_t) { return cudaMalloc(p, n); }
 cudaError_t cudaFreeAsync(void* p, cudaStream_t) { return cudaFree(p); }
 cudaError_t cudaHostAlloc(void** p, size_t n, unsigned) {
-  if (fake::refused()) return cudaErrorStreamCaptureUnsupported;
   fake::count["cudaMallocHost"]++;
+  if (fake::no_pinned) return fake::last_error = cudaErrorMemoryAllocation;
   *p = std::calloc(1, n);
   fake::pinned[(char*)*p] = n;
   return cudaSuccess;
 }
 cudaError_t cudaMallocHost(void** p, size_t n) { return cudaHostAlloc(p, n, 0); }
 cudaError_t cudaFreeHost(void* p) {  // not documented to wait
-  if (fake::refused()) return cudaErrorStreamCaptureUnsupported;
   const size_t n = fake::pinned[(char*)p];
   for (const fake::Op& o : fake::queue)
     if (o.pinned && (const char*)o.src >= (char*)p && (const char*)o.src < (char*)p + n) {
@@ -267,7 +260,6 @@ cudaError_t cudaMemset(void* d, int v, size_t n) {
 }
 
 cudaError_t cudaStreamCreateWithFlags(cudaStream_t* s, unsigned) {
-  if (fake::refused()) return cudaErrorStreamCaptureUnsupported;
   *s = (cudaStream_t) new fake::Stream();
   return cudaSuccess;
 }
@@ -290,12 +282,7 @@ cudaError_t cudaStreamIsCapturing(cudaStream_t s, cudaStreamCaptureStatus* c) {
   *c = fake::of(s)->capture ? cudaStreamCaptureStatusActive : cudaStreamCaptureStatusNone;
   return cudaSuccess;
 }
-cudaError_t cudaThreadExchangeStreamCaptureMode(cudaStreamCaptureMode* m) {
-  std::swap(*m, fake::mode);
-  return cudaSuccess;
-}
 cudaError_t cudaEventCreate(cudaEvent_t* e) {
-  if (fake::refused()) return cudaErrorStreamCaptureUnsupported;
   *e = (cudaEvent_t) new fake::Event();
   return cudaSuccess;
 }
@@ -329,7 +316,7 @@ cudaError_t cudaStreamEndCapture(cudaStream_t s, cudaGraph_t* g) {
   return cudaSuccess;
 }
 cudaError_t cudaGraphInstantiate(cudaGraphExec_t* x, cudaGraph_t g, unsigned long long) {
-  if (fake::refused()) return cudaErrorStreamCaptureUnsupported;
+  if (fake::no_graphs) return fake::last_error = cudaErrorMemoryAllocation;
   *x = (cudaGraphExec_t) new fake::Graph(*(fake::Graph*)g);
   return cudaSuccess;
 }

@@ -178,12 +178,39 @@ static void other_scenes() {
   gs_destroy_scene(s);
 }
 
+// A warmed scene's synchronous calls allocate nothing that they cannot do
+// without: with no memory for a graph or its page-locked table they go on plain.
+static void no_memory_for_graphs() {
+  static float image[4 * 64 * 64];
+  const gs_camera c = camera(64, 64);
+  const gs_pose p = pose(0);
+  double loss, grad[6];
+  for (bool* gone : {&fake::no_pinned, &fake::no_graphs}) {
+    gs_scene* s = scene(100);
+    render(s, c);
+    CHECK(gs_render_pose_grad(s, &c, &p, image, image, nullptr, 1.0f, nullptr, &loss, grad, nullptr) == GS_OK);
+    fake::count.clear();
+    *gone = true;
+    for (int k = 0; k < 40; ++k) {
+      render(s, c);
+      CHECK(gs_render_pose_grad(s, &c, &p, image, image, nullptr, 1.0f, nullptr, &loss, grad, nullptr) == GS_OK);
+    }
+    CHECK(fake::count["replays"] == 0 && fake::count["kernel k_project"] >= 80);
+    *gone = false;
+    for (int k = 0; k < 20; ++k) render(s, c);
+    CHECK(fake::count["replays"] > 0);
+    CHECK(cudaGetLastError() == cudaSuccess);
+    gs_destroy_scene(s);
+  }
+}
+
 int main(int argc, char** argv) {
   const std::map<std::string, void (*)()> all = {{"batches_of_changing_size", batches_of_changing_size},
                                                     {"two_devices", two_devices},
                                                     {"early_starts", early_starts},
                                                     {"sizes_in_pairs", sizes_in_pairs},
-                                                    {"other_scenes", other_scenes}};
+                                                    {"other_scenes", other_scenes},
+                                                    {"no_memory_for_graphs", no_memory_for_graphs}};
   const auto it = all.find(argc > 1 ? argv[1] : "");
   if (it == all.end()) return 2;
   it->second();

@@ -23,7 +23,8 @@ def host_calls(libgsr_path, tmp_path_factory):
     return exe
 
 
-@pytest.mark.parametrize("scenario", ["batches_of_changing_size", "two_devices", "early_starts", "sizes_in_pairs", "other_scenes"])
+@pytest.mark.parametrize("scenario", ["batches_of_changing_size", "two_devices", "early_starts", "sizes_in_pairs", "other_scenes",
+                                      "no_memory_for_graphs"])
 def test_host_calls(host_calls, scenario):
     r = subprocess.run([host_calls, scenario], capture_output=True, text=True, timeout=120)
     assert r.returncode == 0, r.stdout + r.stderr
