@@ -424,11 +424,14 @@ void fill_table(const gs_scene* s, const std::vector<View>& hv, const std::vecto
 }
 
 // The tile counters start at zero: the sort leaves them so, and they are only
-// cleared here when they are new or a call failed on the way there.
+// cleared here when they are new or a call failed on the way there. Under the
+// caller's own capture nothing has run yet: then counts_zero stays false.
 gs_status zero_counts(gs_scene* s, cudaStream_t st) {
   if (s->counts_zero) return GS_OK;
+  cudaStreamCaptureStatus cs;
+  GS_CUDA(cudaStreamIsCapturing(st, &cs));
   GS_CUDA(cudaMemsetAsync(s->tile_ctr.p, 0, ctr_words(s->tile_cap) * sizeof(uint32_t), st));
-  s->counts_zero = true;
+  s->counts_zero = cs == cudaStreamCaptureStatusNone;
   return GS_OK;
 }
 
@@ -495,6 +498,7 @@ gs_status enqueue(gs_scene* s, const std::vector<View>& hv, const std::vector<in
   const int mode = g ? kModeTan : (feats && s->feat_dim) ? kModeFwdFeat : kModeFwd;
   const int grid = s->sm_count * std::max(1, cfg.grid_mult[mode]);  // projection, shading, scatter, sort
   GS_CUDA(mark(0));
+  const bool zero = s->counts_zero;
   if (!graph) s->counts_zero = false;  // until the sort is on the stream
   GS_CUDA(launch_project(sc, dviews, nv, w, grid, st));
   GS_CUDA(mark(1));
@@ -529,7 +533,7 @@ gs_status enqueue(gs_scene* s, const std::vector<View>& hv, const std::vector<in
   GS_CUDA(launch_scatter(dviews, w, grid, st, early));
   GS_CUDA(mark(4));
   GS_CUDA(launch_sort_tiles(w, grid, st, early));
-  if (!graph) s->counts_zero = true;
+  if (!graph) s->counts_zero = zero;
   if (fork) GS_CUDA(cudaStreamWaitEvent(st, s->ev_shade, 0));
   GS_CUDA(mark(5));
   if (!g || feats) GS_CUDA(launch_composite(sc, dviews, nv, w, feats, cfg, s->sm_count, st));

@@ -204,13 +204,37 @@ static void no_memory_for_graphs() {
   }
 }
 
+// A call recorded by the caller's own capture has not run: the tile counters of
+// a new workspace are still cleared by the next call.
+static void callers_capture() {
+  gs_scene* s = scene(100);
+  const gs_camera c = camera(64, 64);
+  const gs_pose p = pose(0);
+  const gs_outputs o{};
+  cudaStream_t st;
+  cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking);
+  cudaGraph_t g;
+  cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal);
+  CHECK(gs_render_async(s, &c, &p, &o, st) == GS_OK);
+  cudaStreamEndCapture(st, &g);
+  const int sets = fake::count["cudaMemsetAsync"];
+  render(s, c);
+  CHECK(fake::count["cudaMemsetAsync"] == sets + 1);
+  render(s, c);
+  CHECK(fake::count["cudaMemsetAsync"] == sets + 1);
+  cudaGraphDestroy(g);
+  cudaStreamDestroy(st);
+  gs_destroy_scene(s);
+}
+
 int main(int argc, char** argv) {
   const std::map<std::string, void (*)()> all = {{"batches_of_changing_size", batches_of_changing_size},
                                                     {"two_devices", two_devices},
                                                     {"early_starts", early_starts},
                                                     {"sizes_in_pairs", sizes_in_pairs},
                                                     {"other_scenes", other_scenes},
-                                                    {"no_memory_for_graphs", no_memory_for_graphs}};
+                                                    {"no_memory_for_graphs", no_memory_for_graphs},
+                                                    {"callers_capture", callers_capture}};
   const auto it = all.find(argc > 1 ? argv[1] : "");
   if (it == all.end()) return 2;
   it->second();

@@ -24,7 +24,7 @@ def host_calls(libgsr_path, tmp_path_factory):
 
 
 @pytest.mark.parametrize("scenario", ["batches_of_changing_size", "two_devices", "early_starts", "sizes_in_pairs", "other_scenes",
-                                      "no_memory_for_graphs"])
+                                      "no_memory_for_graphs", "callers_capture"])
 def test_host_calls(host_calls, scenario):
     r = subprocess.run([host_calls, scenario], capture_output=True, text=True, timeout=120)
     assert r.returncode == 0, r.stdout + r.stderr
