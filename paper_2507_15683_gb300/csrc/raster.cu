@@ -16,6 +16,7 @@
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
+#include "gsr_hit.h"
 #include "gsr_internal.h"
 
 namespace gsr {
@@ -24,14 +25,7 @@ namespace {
 constexpr float kAlphaFloor = 1.0f / 255.0f;
 constexpr float kAlphaCap = 0.99f;
 constexpr float kTCut = 1e-4f;
-constexpr int kWarps = kTileThreads / 32;
-
-// -0.5 (A dx^2 + C dy^2) - B dx dy with one fixed rounding sequence, shared by
-// the forward and backward kernels so that both take identical skip decisions.
-__device__ __forceinline__ float gs_power(float A, float B, float C, float dx, float dy) {
-  const float q = __fmaf_rn(C, __fmul_rn(dy, dy), __fmul_rn(A, __fmul_rn(dx, dx)));
-  return __fmaf_rn(-B, __fmul_rn(dx, dy), __fmul_rn(-0.5f, q));
-}
+static_assert(kWarps == kTileThreads / 32, "a warp per 8 x 4 block of the tile");
 
 // Record centre (float-float: high parts in a.xy, half2 low parts in c.w)
 // relative to the tile origin (X0, Y0): exact subtraction, one rounding.
@@ -263,60 +257,6 @@ __device__ __forceinline__ void warp_block(int tid, int& lx, int& ly, int& bx, i
   by = (warp >> 1) * 4;
   lx = bx + (lane & 7);
   ly = by + (lane >> 3);
-}
-
-// Threshold of the alpha-floor test as an ellipse: o exp(power) >= 1/255 with
-// power = -q/2, q(d) = A dx^2 + 2 B dx dy + C dy^2, needs q <= 2 ln(255 o).
-// Margins (1 % + 0.01 on the log, 0.1 % + 1e-3 on the threshold) cover the
-// fp32 evaluation of the per-pixel test; -1 marks a Gaussian whose opacity
-// cannot reach the floor anywhere.
-__device__ __forceinline__ float floor_threshold(float o) {
-  const float Lp = __logf(255.0f * o) * 1.01f + 0.01f;
-  return Lp > 0.0f ? 2.0f * Lp * 1.001f + 1e-3f : -1.0f;
-}
-
-// Bit w set when a staged Gaussian (centre a.xy in tile-local pixels, conic
-// A = a.z, B = a.w, C) can reach the floor at some pixel centre of warp w's 8 x 4
-// block, for the warps w0 <= w < w1: the minimum over the block of the
-// positive-definite quadratic q is at most thr. If not, every pixel of the warp
-// would skip the Gaussian, so the warp skips it without changing any result.
-// The minimum is q at the centre (0) when the centre is inside, and otherwise
-// lies on an edge that faces the centre: moving from any other point of the
-// block towards the centre lowers q. So a block takes at most two edges, the
-// facing vertical one (whose terms are shared by the four blocks of a column of
-// blocks) and the facing horizontal one (shared by the two of a row). Computed
-// once per staged Gaussian and warp block by a staging thread. Taking the best
-// of all four edges per block, behind a bounding-box test, cost about 450 warp
-// instructions for 32 entries, 12 % of the forward pass: with this and the
-// exponential below, 162 -> 155 us (1080p forward), 452 -> 425 us (tangent pass).
-template <int W0 = 0, int W1 = kWarps>
-__device__ __forceinline__ uint32_t warp_hit_mask(float4 a, float C, float thr, int w0 = W0, int w1 = W1) {
-  if (!(thr > 0.0f)) return 0u;
-  const float A = a.z, B = a.w;
-  if (!(A > 0.0f) || !(C > 0.0f) || !(A * C - B * B > 0.0f)) return (1u << w1) - (1u << w0);
-  const float kx = -__fdividef(B, C), ky = -__fdividef(B, A);  // best dy on a vertical edge per dx, best dx on a horizontal one per dy
-  uint32_t mask = 0u;
-#pragma unroll
-  for (int cx = 0; cx < 2; ++cx) {
-    const float dxl = (float)(8 * cx) + 0.5f - a.x, dxh = dxl + 7.0f;
-    const float fx = dxl > 0.0f ? dxl : fminf(dxh, 0.0f);  // facing vertical edge, 0: the centre is between the edges
-    const float vy = kx * fx, va = A * fx * fx, vb = 2.0f * B * fx;
-#pragma unroll
-    for (int ry = 0; ry < 4; ++ry) {
-      const int wv = 2 * ry + cx;
-      if (wv < w0 || wv >= w1) continue;
-      const float dyl = (float)(4 * ry) + 0.5f - a.y, dyh = dyl + 3.0f;
-      const float fy = dyl > 0.0f ? dyl : fminf(dyh, 0.0f);
-      // on the vertical edge (for fx = 0 this is q at dx = 0: an upper bound of the minimum, and 0 inside)
-      const float y = fminf(fmaxf(vy, dyl), dyh);
-      float best = fmaf(fmaf(C, y, vb), y, va);
-      // on the horizontal edge
-      const float x = fminf(fmaxf(ky * fy, dxl), dxh);
-      best = fminf(best, fmaf(fmaf(A, x, 2.0f * B * fy), x, C * fy * fy));
-      if (best <= thr) mask |= 1u << wv;
-    }
-  }
-  return mask;
 }
 
 // exp of the blending power as 2^(p log2 e). Powers below about -87, whose
