@@ -53,3 +53,43 @@ def test_empty_scene(gsr):
     loss, grad = S.render_pose_grad(cam, np.eye(4), out["rgb"], out["depth"])
     assert loss == 0.0 and not np.any(grad)
     S.close()
+
+
+@pytest.mark.parametrize("what,n,scale,size", [("records", 200000, 1.0, 128), ("pairs", 4000, 12.0, 512)])
+def test_replay_that_outgrows_the_workspace(gsr, what, n, scale, size):
+    # captured and replayed at a pose that sees nothing, on the first guess of the workspace (65,536 records, eight
+    # pairs each); then a replay needs more: the call is done again on a grown workspace, and the tile counters start
+    # at zero afterwards
+    sc = synth.tiny_scene(3, n=n)
+    sc["scales"] = (sc["scales"] * scale).astype(np.float32)
+    cam = synth.camera(size, size, float(size))
+    away = np.diag([-1.0, 1.0, -1.0, 1.0])
+    F = gsr.Scene(sc)
+    want = F.render(cam, np.eye(4))
+    tgt = (torch.full_like(want["rgb"], 0.5), torch.full_like(want["depth"], 5.0))
+    grad = F.render_pose_grad(cam, np.eye(4), *tgt)
+    F.close()
+
+    def render(S):
+        out = S.render(cam, np.eye(4))
+        for k, v in want.items():
+            assert torch.equal(out[k], v), k
+
+    def gradient(S):
+        loss, g = S.render_pose_grad(cam, np.eye(4), *tgt)
+        assert loss == grad[0]
+        np.testing.assert_array_equal(g, grad[1])
+
+    for first, second in ((render, gradient), (gradient, render)):
+        S = gsr.Scene(sc)
+        for _ in range(CALLS):
+            S.render(cam, away)
+            S.render_pose_grad(cam, away, *tgt)
+        assert S.status()[1] == 0
+        first(S)
+        _, records, pairs = S.status()
+        assert records > 65536 if what == "records" else (records < 65536 and pairs > 8 * 65536)
+        for _ in range(CALLS):
+            second(S)
+            first(S)
+        S.close()
