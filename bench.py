@@ -762,7 +762,7 @@ def bench_pmm(gsr, synth, torch, pk_src, steps, warmup, with_oracle=False):
     M.close()
     n = (H // 8) * (W // 8)
     sims = float(n) * n
-    mma_flops = 3 * 2 * 2 * 32 * sims  # three split products, two passes over the tiles, K = 32
+    mma_flops = pmm_tensor_flops(n)
     sm = torch.cuda.get_device_properties(0).multi_processor_count
     mufu_peak = sm * 32 * float(pk.get("sm_max_mhz", 2070.0)) * 1e6  # exp2 per second (32 per SM per clock, measured)
     decisions = pmm_decisions(gsr, synth, torch, scene, T_ref, T_q) if with_oracle else None
@@ -779,6 +779,13 @@ def bench_pmm(gsr, synth, torch, pk_src, steps, warmup, with_oracle=False):
                        "note": "K = 32: the contraction is small; the epilogue (exp, reductions, argmax) bounds"},
             "exp": {"count": int(sims), "achieved_per_s": sims / (ms * 1e-3), "mufu_peak_per_s": mufu_peak,
                     "frac": sims / (ms * 1e-3) / mufu_peak}}
+
+
+def pmm_tensor_flops(n):
+    """Tensor-core operations of a match of n query and n rendered cells: three
+    split products of K = 32 for every similarity, in each of the three passes
+    over the tiles (sums, row argmax, column argmax)."""
+    return 3 * 3 * 2 * 32 * float(n) * n
 
 
 def pmm_decisions(gsr, synth, torch, scene, T_ref, T_q):
