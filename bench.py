@@ -9,7 +9,9 @@ L1 photometric + 0.1 L1 depth loss and its se(3) pose gradient (fp64
 reduction). ``value`` is rendered-and-differentiated Mpix/s (whole job); the
 line also reports forward-only Mpix/s, pose-gradient iterations/s and the
 batched-vs-single-pose factor on the mixed-resolution batch (84 candidate
-poses, 2M Gaussians with 32 BF16 feature channels).
+poses, 2M Gaussians with 32 BF16 feature channels). The full record of every
+section (errors against the oracle, refinement, batches, matching, ...) goes to
+standard error as one JSON object.
 
 L2 is flushed (256 MB write) between timed steps, outside the timed events.
 ``python bench.py [--gpus N --steps K --warmup W] [--impl reference]``; for
@@ -519,7 +521,8 @@ def main():
         "cpu_baseline": cpu,
     }
     if rank == 0:
-        print(json.dumps(line), flush=True)
+        print(json.dumps(line), file=sys.stderr, flush=True)
+        print(json.dumps(short_line(line)), flush=True)
     S.close()
     if world > 1:
         torch.distributed.destroy_process_group()
@@ -779,6 +782,49 @@ def bench_pmm(gsr, synth, torch, pk_src, steps, warmup, with_oracle=False):
                        "note": "K = 32: the contraction is small; the epilogue (exp, reductions, argmax) bounds"},
             "exp": {"count": int(sims), "achieved_per_s": sims / (ms * 1e-3), "mufu_peak_per_s": mufu_peak,
                     "frac": sims / (ms * 1e-3) / mufu_peak}}
+
+
+# sections of the full record, and the numbers of each that the short line keeps
+SECTION_NUMBERS = {
+    "refine_iters_per_s": ("refine", "single", "iters_per_s"),
+    "batched_fwd_speedup": ("batched", "tuned", "forward", "speedup"),
+    "batched_grad_speedup": ("batched", "tuned", "pose_grad", "speedup"),
+    "batched_grad_ms": ("batched", "tuned", "pose_grad", "batched_ms"),
+    "match_ms": ("pmm", "ms"),
+    "visibility_ms": ("visibility", "ms"),
+    "pnp_ms": ("dense", "pnp_ms"),
+    "localisation_ms": ("dense", "algorithm2", "ms_per_localisation"),
+}
+LINE_KEYS = ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better", "scaling",
+             "vs_baseline", "dtype", "data", "config", "clocks", "e2e", "gpu_launches", "untuned",
+             "pose_grad_iters_per_s", "fwd_mpix_s", "fwd_ms", "roofline", "kernels")
+LINE_LIMIT = 2800  # characters
+
+
+def short_line(full):
+    """The line on standard output: the headline with its configuration, clocks,
+    end-to-end figure and roofline, the kernels' times and one number per
+    section, short enough that a log's last few thousand characters hold all of
+    it. The full record goes to standard error."""
+    line = {k: full[k] for k in LINE_KEYS if full.get(k) is not None or k == "vs_baseline"}
+    if full.get("kernels"):
+        line["kernels"] = {k: round(v["ms"], 5) for k, v in full["kernels"].items()}
+    if full.get("cpu_baseline"):
+        line["cpu_baseline"] = {k: full["cpu_baseline"][k] for k in ("value", "unit", "cores", "kind")}
+    sections = {}
+    for name, path in SECTION_NUMBERS.items():
+        v = full
+        for k in path:
+            v = v.get(k) if isinstance(v, dict) else None
+        if v is not None:
+            sections[name] = float("%.5g" % v)
+    line["sections"] = sections
+    line["full_record"] = "standard error"
+    for optional in ("untuned", "kernels", "sections", "roofline"):  # longer than any workload of this file gives
+        if len(json.dumps(line)) <= LINE_LIMIT:
+            break
+        line.pop(optional, None)
+    return line
 
 
 def pmm_tensor_flops(n):
