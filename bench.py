@@ -47,6 +47,7 @@ FLOPS_PER_EVAL = 14
 # directions (5 FMA each) 60, dalpha 6, dw = dalpha T + a dT 18, dT 6, dC 36,
 # colour rows (3 x 3 FMA) 18, dD 24
 FLOPS_PER_BLEND = 180
+JAC_FLOATS = 44  # of a record's pose Jacobian and colour
 # DRAM bytes (read + write) of one tangent-pass launch on this workload, from
 # one ncu capture of this kernel (dram__bytes_read.sum + dram__bytes_write.sum);
 # None whenever the kernel has changed since that capture
@@ -426,7 +427,7 @@ def main():
     # (their data mostly stays in the L2, so these fractions measure latency, not bandwidth)
     n_tiles = tx * ty
     alg_bytes = {"project": 16 * 1_000_000 + 32 * n_rec,       # means of all, covariances of the visible
-                 "shade": n_rec * (48 + 4 * 48 + 64 + 4 * 48),  # record + SH in, record + pose Jacobian out
+                 "shade": n_rec * (48 + 4 * 48 + 64 + 4 * JAC_FLOATS),  # record + SH in, record + pose Jacobian out
                  "scan_tiles": 12 * n_tiles,                     # counts in, offsets and cursors out
                  "scatter": 16 * n_rec + 8 * n_pairs,            # record bounds in, (depth, record) pairs out
                  "sort": 16 * n_pairs}                           # pairs in and out

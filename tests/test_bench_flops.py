@@ -1,4 +1,5 @@
-"""bench.py's operation count of a match, against the passes that csrc/pmm.cu launches and the MMAs of a tile."""
+"""bench.py's operation and byte counts against the code: the passes of a match that csrc/pmm.cu launches and the MMAs
+of a tile, and the size of a Jacobian record."""
 import os
 import re
 
@@ -14,3 +15,8 @@ def test_match_tensor_flops():
     mmas = body[:body.index("\n}")].count("mma_bf16(tmem,")  # each 128 x 128 x 16
     n = 128 * 50
     assert bench.pmm_tensor_flops(n) == passes * (n // 128) ** 2 * mmas * 2 * 128 * 128 * 16
+
+
+def test_jacobian_record_size():
+    src = open(os.path.join(os.path.dirname(PMM), "gsr_internal.h")).read()
+    assert bench.JAC_FLOATS == int(re.search(r"kJacStride = (\d+)", src).group(1))
