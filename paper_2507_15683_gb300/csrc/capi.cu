@@ -105,7 +105,8 @@ struct GraphCache {
   uint64_t used = 0;  // synchronous calls: number of the last one
 };
 constexpr int kSyncGraphs = 8;     // graphs of synchronous calls per scene
-constexpr int kPlainCalls = 8;     // plain calls of a key before it is captured
+constexpr int kPlainRenders = 8;   // plain calls of a key before it is captured
+constexpr int kPlainGrads = 2;
 
 }  // namespace
 
@@ -919,16 +920,16 @@ std::vector<char> graph_key(const std::vector<View>& hv, const GradIn* g) {
 
 // A synchronous single-view call replayed from a CUDA graph: one launch instead
 // of the call's table upload, six to seven kernel launches, events and
-// read-backs. A capture costs about as much as eight replays save (a 128 x 128
-// render of 1,000 Gaussians: plain 56 us, the call that captures 125, replayed
-// 47; its gradient 105, 165 and 75), so a key is captured at its ninth call: a
-// scene that is rendered a few times, or in sizes that hardly come back, pays
-// nothing, and one whose sizes return waits for the capture once in nine calls
-// at the most. kSyncGraphs keys are kept, the one not used for longest gives
-// way. A call that overflows the workspace is redone by the regrow path, and its
-// key counts plain calls again; so does one whose workspace or launch
-// configuration changed, or whose capture failed. With kernel timing on, the ordinary path runs (graphs
-// carry no timing events).
+// read-backs. A capture costs what eight replayed renders or two to three
+// replayed gradients save (a 128 x 128 render of 1,000 Gaussians: plain 56 us,
+// the call that captures 125, replayed 47; its gradient 105, 165 and 75), so a
+// key is captured after that many plain calls: a scene that is rendered a few
+// times, or in sizes that hardly come back, pays nothing, and one whose sizes
+// return waits for a capture at most that often. kSyncGraphs keys are kept, the
+// one not used for longest gives way. A call that overflows the workspace is
+// redone by the regrow path, and its key counts plain calls again; so does one
+// whose workspace or launch configuration changed, or whose capture failed. With
+// kernel timing on, the ordinary path runs (graphs carry no timing events).
 gs_status run_sync_graphed(gs_scene* s, const std::vector<View>& hv, uint64_t n_tiles, const GradIn* g,
                            cudaStream_t st) {
   if (s->timing || hv.size() != 1 || (g && g->result)) return run_sync(s, hv, n_tiles, g, st);
@@ -952,7 +953,7 @@ gs_status run_sync_graphed(gs_scene* s, const std::vector<View>& hv, uint64_t n_
       G->valid = false;
       G->plain = 0;
     }
-    if (G->plain < kPlainCalls) {
+    if (G->plain < (g ? kPlainGrads : kPlainRenders)) {
       ++G->plain;
       return run_sync(s, hv, n_tiles, g, st);
     }

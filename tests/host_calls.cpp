@@ -124,8 +124,9 @@ static void render(gs_scene* s, const gs_camera& c) {
   CHECK(gs_render(s, &c, &p, &o, nullptr) == GS_OK);
 }
 
-// Synchronous renders are captured once their size has come up often, and only
-// once: not again for a size that comes back, and never for sizes that are many.
+// Synchronous calls are captured once their size has come up often enough (a
+// gradient, whose replay saves more, sooner), and only once: not again for a size
+// that comes back, and never for sizes that are many.
 static void sizes_in_pairs() {
   gs_scene* s = scene(100);
   fake::count.clear();
@@ -145,6 +146,16 @@ static void sizes_in_pairs() {
       gs_destroy_scene(t);
     }
   CHECK(fake::count["captures"] == 2);
+  static float image[4 * 64 * 64];
+  const gs_camera c = camera(64, 64);
+  const gs_pose p = pose(0);
+  double loss, grad[6];
+  for (int k = 0; k < 5; ++k) {
+    const int before = fake::count["replays"];
+    CHECK(gs_render_pose_grad(s, &c, &p, image, image, nullptr, 1.0f, nullptr, &loss, grad, nullptr) == GS_OK);
+    CHECK(fake::count["replays"] == before + (k >= 2));
+  }
+  CHECK(fake::count["captures"] == 3);
   gs_destroy_scene(s);
 }
 
