@@ -120,8 +120,10 @@ gs_status gs_scene_reserve(gs_scene* scene, int64_t max_records, int64_t max_pai
 
 /* Render one view (Sec. 3.1 rasterization at the pose of Sec. 3.4).
  * Synchronous: waits for the stream, and when the workspace was too small
- * grows it and renders again, so the outputs are complete on return.
- * Errors: INVALID_ARG, OOM, CUDA. */
+ * grows it and renders again, so the outputs are complete on return. (CUDA
+ * refuses that wait while another thread captures in global mode;
+ * gs_render_noalloc makes none.) A size that comes up often is replayed from a
+ * CUDA graph. Errors: INVALID_ARG, OOM, CUDA. */
 gs_status gs_render(gs_scene* scene, const gs_camera* cam, const gs_pose* pose, const gs_outputs* out,
                     void* stream);
 

@@ -87,12 +87,14 @@ struct SceneDev {
 // spreads them over more 32-byte sectors: the L2 performs atomics on one sector
 // one after another, and with eight counters in each the 2,040 tiles of a
 // 960 x 540 view queued on 255 sectors. The shift is the largest (at most one
-// counter per sector) that keeps the array within kCtrWords; from there on the
-// sectors are plenty and the scan, one block, would pay for the width. Measured
-// with strides of 1 / 2 / 4 / 8 words: projection and scatter of a 960 x 540 view
+// counter per sector) that keeps the array within kCtrWords. Measured with
+// strides of 1 / 2 / 4 / 8 words: projection and scatter of a 960 x 540 view
 // (500,000 Gaussians, 311,000 pairs) 24.6 + 16.5 / 17.1 + 14.6 / 12.9 + 9.9 /
 // 13.7 + 8.6 us; of a 3840 x 2160 view (3 M, 9.1 M pairs) 73 + 104 / 65 + 101 /
-// 69 + 107 / 79 + 116 us, its scan 22 / 23 / 33 / 47 us.
+// 69 + 107 / 79 + 116 us, its scan (one block, which pays for the width) 22 / 23 /
+// 33 / 47 us. There the limit picks stride 1, 199 us in all, although stride 2
+// takes 189, 0.3 % of that view's gradient: the limit was set for the sizes below
+// and has not been swept above them.
 constexpr uint32_t kCtrWords = 32768;
 constexpr int ctr_shift(uint64_t n_tiles) {
   int s = 0;

@@ -235,11 +235,13 @@ __device__ __forceinline__ void eval_sh_deg(int deg, const float4* shp, float x,
 // Bound by the atomics that count the pairs (their spread over the L2's sectors:
 // ctr_shift) and by latency: a warp has one or two chunks. With the views read
 // from the call table instead of shared memory (about twenty words per chunk and
-// view) and every rectangle walked by its own lane, 16 views of 2 M Gaussians
-// took 362 us, now 235 to 255; one 1080p view of 1 M took 31 us, now 23; one
-// 960 x 540 view of 500,000 took 24.6 us, now 14. Blocks per SM: 64 registers and
-// 4 blocks; 5 and 6 blocks (48 and 40 registers, with spills) took 32 and 38 us at
-// 1080p against 27.
+// view), every rectangle walked by its own lane and eight counters to a sector,
+// 16 views of 2 M Gaussians took 362 us, now 234; one 1080p view of 1 M took 31
+// us, now 21; one 960 x 540 view of 500,000 took 24.6 us, now 12 (traces of
+// repeated calls; after an L2 flush or under ncu the 1080p view takes 23 to 24).
+// Blocks per SM: 64 registers and 4 blocks; 5 and 6 blocks (48 and 40 registers,
+// with spills) took 32 and 38 us at 1080p against 27, before the record counters
+// were spread too.
 // ---------------------------------------------------------------------------
 constexpr int kProjResident = 4;       // blocks per SM
 constexpr unsigned kSoloTiles = 12u;   // tiles that a lane counts by itself; the warp shares a larger rectangle

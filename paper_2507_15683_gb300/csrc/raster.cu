@@ -919,13 +919,13 @@ Variant variant() {
   return {k_composite<FEAT, TAN, KB, MINB>, comp_smem<FEAT, TAN, KB>(), KB, MINB};
 }
 const Variant* variant_table(int mode) {
-  // forward: 64 registers for 4 CTAs per SM beat 48 (spilling) for 5: 285 against 300 us for the 1080p call
+  // forward: 64 registers for 4 CTAs per SM beat 48 (spilling) for 5: 264 against 275 us for repeated 1080p calls
   static const Variant fwd[kCompVariants] = {variant<0, false, 256, 4>(), variant<0, false, 128, 5>(),
                                              variant<0, false, 256, 5>(), variant<0, false, 64, 5>()};
   static const Variant feat[kCompVariants] = {variant<32, false, 256, 3>(), variant<32, false, 128, 3>(),
                                               variant<32, false, 128, 4>(), variant<32, false, 64, 4>()};
-  // tangent: 80 registers for 3 CTAs beat 64 (spilling) for 4: 657 against 669 us for the 1080p gradient, 8,071
-  // against 8,285 us for 50 refinement steps at 960 x 540, 3,662 against 3,689 us at 3840 x 2160
+  // tangent: 80 registers for 3 CTAs beat 64 (spilling) for 4: 660 against 671 us for repeated 1080p gradients, 8,044
+  // against 8,315 us for 50 refinement steps at 960 x 540, 3,663 against 3,691 us at 3840 x 2160
   static const Variant tan[kCompVariants] = {variant<0, true, 128, 3>(), variant<0, true, 64, 4>(),
                                              variant<0, true, 128, 4>(), variant<0, true, 64, 3>()};
   return mode == kModeTan ? tan : mode == kModeFwdFeat ? feat : fwd;
