@@ -121,9 +121,9 @@ gs_status gs_scene_reserve(gs_scene* scene, int64_t max_records, int64_t max_pai
 /* Render one view (Sec. 3.1 rasterization at the pose of Sec. 3.4).
  * Synchronous: waits for the stream, and when the workspace was too small
  * grows it and renders again, so the outputs are complete on return. (CUDA
- * refuses that wait while another thread captures in global mode;
- * gs_render_noalloc makes none.) A size that comes up often is replayed from a
- * CUDA graph. Errors: INVALID_ARG, OOM, CUDA. */
+ * refuses that wait, and breaks the other capture, while another thread captures
+ * in global mode; this holds for every synchronous call.) A size that comes up
+ * often is replayed from a CUDA graph. Errors: INVALID_ARG, OOM, CUDA. */
 gs_status gs_render(gs_scene* scene, const gs_camera* cam, const gs_pose* pose, const gs_outputs* out,
                     void* stream);
 
@@ -442,11 +442,9 @@ gs_status gs_visibility(gs_scene* scene, const gs_camera* cam, const gs_pose* po
  *
  * Why: some callers cannot ask the CUDA allocator for memory when they render
  * -- a service that sized its device memory once at start-up and may not grow
- * it per request, a plug-in whose host application owns every device
- * allocation, or code that runs while another thread captures a CUDA graph in
- * global mode, where cudaMalloc is not permitted. gs_render needs a scene
- * (created with cudaMalloc) and grows its workspace on demand; this entry
- * point needs neither.
+ * it per request, or a plug-in whose host application owns every device
+ * allocation. gs_render needs a scene (created with cudaMalloc) and grows its
+ * workspace on demand; this entry point needs neither.
  *
  * What: renders one view exactly like gs_render (same kernels, same results),
  * reading the Gaussians straight from the caller's device arrays in desc
@@ -462,7 +460,8 @@ gs_status gs_visibility(gs_scene* scene, const gs_camera* cam, const gs_pose* po
  * the device; the outputs are then incomplete).
  *
  * Calls no cudaMalloc, cudaFree or allocating library routine. Synchronous:
- * waits for the stream to read the device counters. The first call on a device
+ * waits for the stream to read the device counters, so that CUDA refuses it, like
+ * gs_render, while another thread captures in global mode. The first call on a device
  * looks up the array's device address (cudaGetSymbolAddress) for that device;
  * make that first call before any stream capture. All calls share the one
  * array: calls whose work overlaps on the GPU (different streams or host
